@@ -61,10 +61,9 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : 3)
     pdl_enter();
     constexpr int SPC = 256 / (B * B / 4);
     const int n = *pn;
-    for (int i0 = blockIdx.x * SPC; i0 < n; i0 += gridDim.x * SPC) {  // grid stride (vec_grid)
-        fused_v4_task<S, C, B, COLL, true>(P, list, n, i0, fin, fout, ffine, level, allow_force);
-        __syncthreads();  // the task's neighbour table is rewritten by the next one
-    }
+    int pass = 0;
+    for (int i0 = blockIdx.x * SPC; i0 < n; i0 += gridDim.x * SPC)  // grid stride (vec_grid)
+        fused_v4_task<S, C, B, COLL, true>(P, list, n, i0, pass++, fin, fout, ffine, level, allow_force);
 }
 
 // Thread blocks of a vector-kernel launch: at most `waves` waves of resident
@@ -96,10 +95,9 @@ __global__ void __launch_bounds__(256, 3)
     pdl_enter();
     constexpr int SPC = 256 / (B * B / 8);
     const int n = *pn;
-    for (int i0 = blockIdx.x * SPC; i0 < n; i0 += gridDim.x * SPC) {  // grid stride (vec_grid)
-        fused_v8_task<S, C, B, COLL, true, SH>(P, list, n, i0, fin, fout, ffine, level, allow_force);
-        __syncthreads();  // the task's neighbour table is rewritten by the next one
-    }
+    int pass = 0;
+    for (int i0 = blockIdx.x * SPC; i0 < n; i0 += gridDim.x * SPC)  // grid stride (vec_grid)
+        fused_v8_task<S, C, B, COLL, true, SH>(P, list, n, i0, pass++, fin, fout, ffine, level, allow_force);
 }
 
 // collision only, on pre-collision populations (the state at t = 0)

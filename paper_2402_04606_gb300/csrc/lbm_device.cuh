@@ -877,15 +877,18 @@ __device__ __forceinline__ uint4 ld_u4(const uint4* p) {
 // non-periodic side (per warp: a warp never spans two blocks) take the scalar
 // path above.
 // The kernel's work for the list items item0, item0 + 1, ... (one per
-// B * B / 4 threads of the thread block; items from n on are skipped).
+// B * B / 4 threads of the thread block; items from n on are skipped).  pass:
+// counts a block's consecutive calls (its parity picks the neighbour table).
 // NC: the input buffer does not change during the launch (loads may take the
 // read-only path).  Contains a block-wide barrier.
 template <class S, class C, int B, int COLL, bool NC>
-__device__ __forceinline__ void fused_v4_task(const DevPool& P, const int* list, int n, int item0, const S* fin, S* fout,
+__device__ __forceinline__ void fused_v4_task(const DevPool& P, const int* list, int n, int item0, int pass, const S* fin, S* fout,
                                               const S* ffine, int level, int allow_force, S* fhalo = nullptr) {
     static_assert(sizeof(S) >= 4, "16-bit storage takes the 8-cell kernel");
     constexpr int BB = B * B, TPS = BB / 4, TPR = B / 4;
-    __shared__ int nb[STEP_MAX_THREADS / TPS][9];
+    // two copies: a warp still reading this pass's while another starts the next pass
+    __shared__ int nb2[2][STEP_MAX_THREADS / TPS][9];
+    int(*const nb)[9] = nb2[pass & 1];
     const int ls = threadIdx.x / TPS, t = threadIdx.x % TPS;
     const int item = item0 + ls;
     if (t < 9) nb[ls][t] = item < n ? P.nbr[list[item] * 9 + t] : -1;
@@ -1046,11 +1049,13 @@ __device__ __forceinline__ float el8(const uint4& r, int k) {
 // B * B / 8 threads; n and NC as for fused_v4_task).  Contains a block-wide
 // barrier.
 template <class S, class C, int B, int COLL, bool NC, bool SH>
-__device__ __forceinline__ void fused_v8_task(const DevPool& P, const int* list, int n, int item0, const S* fin, S* fout,
+__device__ __forceinline__ void fused_v8_task(const DevPool& P, const int* list, int n, int item0, int pass, const S* fin, S* fout,
                                               const S* ffine, int level, int allow_force, S* fhalo = nullptr) {
     static_assert(sizeof(S) == 2, "the 8-cell kernel is for 16-bit storage");
     constexpr int BB = B * B, TPS = BB / 8, TPR = B / 8;
-    __shared__ int nb[STEP_MAX_THREADS / TPS][9];
+    // two copies: a warp still reading this pass's while another starts the next pass
+    __shared__ int nb2[2][STEP_MAX_THREADS / TPS][9];
+    int(*const nb)[9] = nb2[pass & 1];
     const int ls = threadIdx.x / TPS, t = threadIdx.x % TPS;
     const int item = item0 + ls;
     if (t < 9) nb[ls][t] = item < n ? P.nbr[list[item] * 9 + t] : -1;

@@ -72,22 +72,43 @@ __device__ __forceinline__ int fused_items(bool vec, int T) {
     return vec ? T / (B * B / CPT) : (T >= B * B ? T / (B * B) : 1);
 }
 
-// list items per round (per) and rounds per task of fused phase ph with n
-// items: a bulk task, and a critical one whose phase would otherwise hand
-// out more than 8 tasks per thread block (a whole level of a large grid, as
-// in the later steps of a launch), take bulk_rounds thread-block fillings;
-// another critical one at most crit_items items (so that a short sweep other
-// phases wait for spreads over more SMs)
-template <class S, int B>
-__device__ __forceinline__ void task_shape(const StepArgs& A, const StepPhase& ph, int n, bool vec, int T, int& per,
-                                           int& rounds) {
-    per = fused_items<S, B>(vec, T);
-    rounds = 1;
-    if (ph.bulk || (long long)n > 8LL * per * gridDim.x) {
-        rounds = A.bulk_rounds;
-        return;
+// How fused phase ph with n items is cut into tasks: `per` items per round and
+// `rounds` rounds per task, or (parts > 1) every item into `parts` tasks of its
+// own.  Handing out a task costs some microseconds of dependent L2 round
+// trips, so a task holds as many items as fill the thread block, and a bulk
+// task (or one of a list of more than 8 fillings of every thread block) up to
+// bulk_rounds fillings: as many as give every thread block the same number of
+// tasks.  crit_items caps a critical task's items (a short sweep other phases
+// wait for).  In FP64 the pipe is the bound (a 16 x 16 item keeps one SM busy for
+// 11 us), so there a short list is spread over every SM, in parts of an item
+// when it has fewer items than half the thread blocks.
+// Measured against bulk tasks of a fixed 8 rounds, us per step: 128^2 in FP64
+// (64 items: 8 tasks on 152 SMs) 41.9 -> 13.1; 2960 x 1488 with the LES
+// collision in FP32 (538 tasks for 456 thread blocks, two unequal waves) 92 ->
+// 71; a 1120 x 640 level of 16-bit blocks (15 tasks of up to 145 us each) in a
+// pitching section's step 117 -> 103.  Spreading short FP32 lists over every SM
+// as well measured slower (a D = 40 cylinder's step 64 -> 86): there the hand-out
+// is the cost.
+struct TaskShape {
+    int per, rounds, parts;
+    __device__ __forceinline__ int tasks(int n) const {
+        return parts > 1 ? n * parts : (n + per * rounds - 1) / (per * rounds);
     }
-    if (A.crit_items > 0 && A.crit_items < per) per = A.crit_items;
+};
+template <class S, int B>
+__device__ __forceinline__ TaskShape task_shape(const StepArgs& A, const StepPhase& ph, int n, bool vec, int T) {
+    TaskShape t{fused_items<S, B>(vec, T), 1, 1};
+    const int grid = gridDim.x;
+    const long long fill = (long long)t.per * grid;  // items of one filling of every thread block
+    if (ph.bulk || n > 8 * fill) {
+        const long long waves = (n + fill * A.bulk_rounds - 1) / (fill * A.bulk_rounds);
+        t.rounds = (int)((n + fill * waves - 1) / (fill * waves));
+    } else if (A.crit_items > 0 && A.crit_items < t.per) {
+        t.per = A.crit_items;
+    }
+    if (sizeof(S) == 8 && n < fill) t.per = (n + grid - 1) / grid;
+    if (sizeof(S) == 8 && !vec && 2LL * n <= grid) t.parts = 4LL * n <= grid ? 4 : 2;
+    return t;
 }
 
 // tasks of phase p at this launch (from the device list lengths)
@@ -97,9 +118,7 @@ __device__ int step_ntasks(const DevPool& P, const StepArgs& A, const StepPhase&
     if (n <= 0) return 0;
     switch (ph.kind) {
     case PH_FUSED: {
-        int per, rounds;
-        task_shape<S, B>(A, ph, n, fused_vec<S, B>(A, ph, n, P.coll), T, per, rounds);
-        return (n + per * rounds - 1) / (per * rounds);
+        return task_shape<S, B>(A, ph, n, fused_vec<S, B>(A, ph, n, P.coll), T).tasks(n);
     }
     case PH_C2F: {
         const int per = T >= B * B ? T / (B * B) : 1;
@@ -141,17 +160,21 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
     S* fhalo = ph.fold ? step_buf<S>(A, ph.ffine) : nullptr;  // the coarse-to-fine copy rides on this sweep
     const int T = blockDim.x;
     const bool vec = fused_vec<S, B>(A, ph, n, P.coll);
-    int per, rounds;
-    task_shape<S, B>(A, ph, n, vec, T, per, rounds);
-    if (!ph.bulk && rounds == 1 && !vec && per <= STEP_META_MAX && per <= T / 32) {
-        const int i0 = local * per, ne = min(n, i0 + per), w = threadIdx.x >> 5;
+    const TaskShape sh = task_shape<S, B>(A, ph, n, vec, T);
+    const int per = sh.per, rounds = sh.rounds;
+    if (rounds == 1 && !vec && per <= STEP_META_MAX && per <= T / 32) {
+        const int i0 = sh.parts > 1 ? local / sh.parts : local * per, ne = min(n, i0 + per), w = threadIdx.x >> 5;
+        // its cells: those of its items, or a part of one item's
+        const int len = sh.parts > 1 ? B * B / sh.parts : (ne - i0) * B * B;
+        const int c0 = sh.parts > 1 ? (local - i0 * sh.parts) * len : 0;
         if (i0 + w < ne) load_meta(P, list[i0 + w], meta[w]);
         if (!gate(true)) return;
-        for_cells(ne, i0, per, B * B, [&](int item, int cell) {
-            const SlotMeta& m = meta[item - i0];
+        for (int c = c0 + threadIdx.x; c < c0 + len; c += T) {
+            const SlotMeta& m = meta[c / (B * B)];
+            const int cell = c % (B * B);
             fused_cell<S, C, COLL, false, MetaS>(P, MetaS{&m}, fin, fout, ffine, m.type, P.inst[m.inst], ph.level,
                                                  cell % B, cell / B, ph.allow_force != 0, fhalo);
-        });
+        }
         return;
     }
     if (!gate(false)) return;
@@ -162,10 +185,10 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
         if constexpr (B >= 16) {
             if (vec) {
                 if constexpr (sizeof(S) == 2)
-                    fused_v8_task<S, C, B, COLL, false, true>(P, list, ne, i0, fin, fout, ffine, ph.level,
+                    fused_v8_task<S, C, B, COLL, false, true>(P, list, ne, i0, r, fin, fout, ffine, ph.level,
                                                               ph.allow_force, fhalo);
                 else
-                    fused_v4_task<S, C, B, COLL, false>(P, list, ne, i0, fin, fout, ffine, ph.level, ph.allow_force,
+                    fused_v4_task<S, C, B, COLL, false>(P, list, ne, i0, r, fin, fout, ffine, ph.level, ph.allow_force,
                                                         fhalo);
                 continue;
             }

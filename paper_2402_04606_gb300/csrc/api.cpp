@@ -47,7 +47,7 @@ struct HostBody {
 //   GF     fine-side halo blocks (coarse-to-fine copy)
 //   GC     coarse-side mailbox blocks (no launch of their own: the coarse
 //          pull merges the fine values; the list keeps their membership)
-//   INDEP  fused blocks that need neither a mailbox nor a force patch
+//   INDEP  fused blocks that need no mailbox and hold no cell a body forces
 //   DEP    the other interior blocks
 //   IBM    instances whose finest level this is
 // Lists are unordered: every block of a launch is independent of the others.
@@ -1051,9 +1051,10 @@ sbot_status build_topology(sbot_ctx* c, int ii, long long n, bool transfer) {
     }
     I.ip.latmap = I.d_latmap;
     if (first) TRY(upload(c, c->d_ip + ii, &I.ip, sizeof(InstParams)));
-    // interior blocks that must wait: a mailbox neighbour (coarse side of an
-    // interface), or, on the finest level, the force patch of the body (every
-    // finest block for a moving body; the stencil box for a static one)
+    // interior blocks in the lists of their own: those with a mailbox neighbour
+    // (coarse side of an interface), which wait for the finer level, and on the
+    // finest level those a body may force (every finest block for a moving body;
+    // the stencil box for a static one), which the IBM waits for
     int bx0 = 1 << 30, by0 = 1 << 30, bx1 = -(1 << 30), by1 = -(1 << 30);
     const bool static_body = I.has_body && I.body.motion == 0;
     if (static_body) {
@@ -1227,9 +1228,9 @@ void drop_graph(sbot_ctx* c, int g) {
 
 // One substep of level l of every instance of group g (m = g + 1 levels) and,
 // recursively, two of every finer level: Algorithm 1 with each stream+collide
-// pair fused into one pull kernel, on the group's stream.  Blocks that need
-// neither a finer level nor the IBM run on a side stream from the start of
-// the substep.  Launch sizes are the list capacities; the kernels read the
+// pair fused into one pull kernel, on the group's stream; then the IBM of the
+// level's bodies.  Blocks that need no finer level and no body forces run on a
+// side stream from the start of the substep.  Launch sizes are the list capacities; the kernels read the
 // current lengths on the device.
 void advance(sbot_ctx* c, const DevPool& P, int g, int l) {
     const int storage = c->storage, gl = gl_of(g + 1, l);
@@ -1258,7 +1259,7 @@ void advance(sbot_ctx* c, const DevPool& P, int g, int l) {
         {
             ProfScope ps(c, 0, gl, LK_INDEP, sd);
             launch_fused(storage, P, lptr(c, gl, LK_INDEP), cptr(c, gl, LK_INDEP), Wi.cap, Wi.cap, c->vec_min_cells, c->staged, cur,
-                         nxt, fine, l, sd, 0);
+                         nxt, fine, l, sd);
         }
         if (!serial) cudaEventRecord(c->ev_join[gl], sd);
     }
@@ -1272,12 +1273,29 @@ void advance(sbot_ctx* c, const DevPool& P, int g, int l) {
         advance(c, P, g, l + 1);
         advance(c, P, g, l + 1);
     }
+    if (fork) {
+        {
+            // below the finest level these are the blocks next to the finer
+            // region: their pulls merge fine values cell by cell, so they take
+            // the one-cell-per-thread kernel whatever their number
+            ProfScope ps(c, 0, gl, LK_DEP, st);
+            launch_fused(storage, P, lptr(c, gl, LK_DEP), cptr(c, gl, LK_DEP), Wd.cap, Wd.cap,
+                         l < g ? -1 : c->vec_min_cells, c->staged, cur, nxt, fine, l, st, fold);
+        }
+        if (!serial) cudaStreamWaitEvent(st, c->ev_join[gl], 0);
+    } else {
+        const WorkList& Wf = W_of(c, gl, LK_FUSED);
+        ProfScope ps(c, 0, gl, LK_FUSED, st);
+        launch_fused(storage, P, lptr(c, gl, LK_FUSED), cptr(c, gl, LK_FUSED), Wf.cap, Wf.cap,
+                     l < g ? -1 : c->vec_min_cells, c->staged, cur, nxt, fine, l, st, fold);
+    }
+    // the bodies on this level: after the sweep, whose unforced cells the IBM collides again with their force
     const WorkList& Wb = W_of(c, gl, LK_IBM);
     if (Wb.cap > 0) {
         if ((c->moving >> g) & 1) cudaStreamWaitEvent(st, c->ev_pose[g], 0);
         {
             ProfScope ps(c, 3, gl, LK_IBM, st);
-            launch_ibm(storage, P, lptr(c, gl, LK_IBM), cptr(c, gl, LK_IBM), Wb.cap, cur, l, 0, c->ibm_smem[g], st, 1,
+            launch_ibm(storage, P, lptr(c, gl, LK_IBM), cptr(c, gl, LK_IBM), Wb.cap, cur, nxt, l, 0, c->ibm_smem[g], st, 1,
                        c->ibm_threads);
         }
         if (--c->ibm_left[g] == 0) {  // the coarse step's last IBM: its force sums run beside the rest
@@ -1287,22 +1305,6 @@ void advance(sbot_ctx* c, const DevPool& P, int g, int l) {
             launch_force_sum(storage, P, lptr(c, gl, LK_IBM), cptr(c, gl, LK_IBM), Wb.cap, 1 << g, sp);
             cudaEventRecord(c->ev_fsum[g], sp);
         }
-    }
-    if (fork) {
-        {
-            // below the finest level these are the blocks next to the finer
-            // region: their pulls merge fine values cell by cell, so they take
-            // the one-cell-per-thread kernel whatever their number
-            ProfScope ps(c, 0, gl, LK_DEP, st);
-            launch_fused(storage, P, lptr(c, gl, LK_DEP), cptr(c, gl, LK_DEP), Wd.cap, Wd.cap,
-                         l < g ? -1 : c->vec_min_cells, c->staged, cur, nxt, fine, l, st, 1, fold);
-        }
-        if (!serial) cudaStreamWaitEvent(st, c->ev_join[gl], 0);
-    } else {
-        const WorkList& Wf = W_of(c, gl, LK_FUSED);
-        ProfScope ps(c, 0, gl, LK_FUSED, st);
-        launch_fused(storage, P, lptr(c, gl, LK_FUSED), cptr(c, gl, LK_FUSED), Wf.cap, Wf.cap,
-                     l < g ? -1 : c->vec_min_cells, c->staged, cur, nxt, fine, l, st, 1, fold);
     }
     c->par[l] ^= 1;
 }
@@ -1352,13 +1354,15 @@ void advance_all(sbot_ctx* c) {
 //   coarse-to-fine copy into level l+1: the last sweep of level l (the coarse
 //     post-collision state it copies, and the merge that read the halo it
 //     overwrites);
-//   IBM of a finest sub-step: the level's previous sweep (the pre-collision
-//     state it pulls) and, for a moving body, the geometry of that step;
-//   sweep of level l, blocks needing no finer level and no force (A): the
-//     level's previous sweep (neighbours; the buffer it overwrites) and the
-//     copy into level l (halo cells);
-//   the other blocks (B): the same, plus the IBM of the sub-step and the two
-//     sweeps of level l+1 (whose halo values the coarse pull merges).
+//   sweep of level l, blocks needing no finer level and away from a body's
+//     stencils (A): the level's previous sweep (neighbours; the buffer it
+//     overwrites) and the copy into level l (halo cells);
+//   the other blocks (B): the same, plus the level's previous IBM (the cells it
+//     collided) and the two sweeps of level l+1 (whose halo values the coarse
+//     pull merges);
+//   IBM of a finest sub-step: whatever B waits for (the pre-collision state it
+//     pulls) and, for a moving body, the geometry of that step; its stores wait
+//     for B, whose unforced values they replace.
 struct PhaseEmit {
     sbot_ctx* c;
     int g;
@@ -1370,14 +1374,14 @@ struct PhaseEmit {
     std::vector<int> geom;
 
     int add(int kind, int level, int gl, int lk, std::initializer_list<int> deps, int fin = -1, int fout = -1,
-            int ffine = -1, int allow_force = 0, int arg = 0) {
+            int ffine = -1, int arg = 0) {
         const WorkList& W = W_of(c, gl, lk);
         if (W.cap <= 0) return -1;
         StepPhase p{};
         p.kind = kind;
         p.bulk = 0;
         p.level = level;
-        p.allow_force = allow_force;
+        p.after = -1;
         p.fin = fin;
         p.fout = fout;
         p.ffine = ffine;
@@ -1409,23 +1413,29 @@ struct PhaseEmit {
             adv(l + 1);
             adv(l + 1);
         }
-        int ibm = -1;
-        if (l == g && bodies) {
-            ibm = add(PH_IBM, l, gl, LK_IBM,
-                      {lastA[l], lastB[l], moving ? geom[n_ibm] : -1, n_ibm == 0 ? prev_fsum : -1}, cur);
-            n_ibm++;
-            last_ibm = ibm;
-        }
         const int c2 = l > 0 ? c2f_into[l] : -1;
         const int fa = l < g ? lastA[l + 1] : -1, fb = l < g ? lastB[l + 1] : -1;
+        const int forced = l == g ? last_ibm : -1;  // the level's previous IBM wrote the cells this sweep pulls
         int A = -1, Bp;
         if (fork) {
-            A = add(PH_FUSED, l, gl, LK_INDEP, {lastA[l], lastB[l], c2}, cur, nxt, fine, 0);
-            Bp = add(PH_FUSED, l, gl, LK_DEP, {lastA[l], lastB[l], c2, ibm, fa, fb}, cur, nxt, fine, 1,
+            // (blocks away from a static body's stencils neither pull nor overwrite a cell that the IBM touches)
+            A = add(PH_FUSED, l, gl, LK_INDEP, {lastA[l], lastB[l], c2, moving ? forced : -1}, cur, nxt, fine);
+            Bp = add(PH_FUSED, l, gl, LK_DEP, {lastA[l], lastB[l], c2, forced, fa, fb}, cur, nxt, fine,
                      l < g ? 1 : 0);  // next to the finer region: one cell per thread
         } else {
-            Bp = add(PH_FUSED, l, gl, LK_FUSED, {lastA[l], lastB[l], c2, ibm, fa, fb}, cur, nxt, fine, 1,
+            Bp = add(PH_FUSED, l, gl, LK_FUSED, {lastA[l], lastB[l], c2, forced, fa, fb}, cur, nxt, fine,
                      l < g ? 1 : 0);
+        }
+        if (l == g && bodies && Bp >= 0) {
+            // it may start when the sweep may (it waits for whatever the
+            // sweep waits for), and waits for the sweep before its stores
+            ph[Bp].bulk = -1;
+            const int ibm = add(PH_IBM, l, gl, LK_IBM,
+                                {lastA[l], lastB[l], c2, last_ibm, moving ? geom[n_ibm] : -1,
+                                 n_ibm == 0 ? prev_fsum : -1}, cur, nxt, -1, n_ibm);
+            ph[ibm].after = Bp;
+            n_ibm++;
+            last_ibm = ibm;
         }
         if (fold && Bp >= 0) {
             ph[Bp].fold = 1;
@@ -1454,10 +1464,10 @@ struct PhaseEmit {
             if (moving) {
                 const int pose = add(PH_POSE, g, glb, LK_IBM, {last_ibm});
                 for (int i = 0; i < (1 << g); i++)
-                    geom.push_back(add(PH_GEOM, g, glb, LK_IBM, {pose}, -1, -1, -1, 0, i));
+                    geom.push_back(add(PH_GEOM, g, glb, LK_IBM, {pose}, -1, -1, -1, i));
             }
             adv(0);
-            if (bodies) prev_fsum = add(PH_FSUM, g, glb, LK_IBM, {last_ibm}, -1, -1, -1, 0, 1 << g);
+            if (bodies) prev_fsum = add(PH_FSUM, g, glb, LK_IBM, {last_ibm}, -1, -1, -1, 1 << g);
         }
     }
 };
@@ -1497,11 +1507,21 @@ bool build_step_phases(sbot_ctx* c, std::vector<StepPhase>& out, int steps) {
         where[r.g][r.i] = (int)out.size();
         StepPhase p = em[r.g].ph[r.i];
         for (int k = 0; k < p.ndep; k++) p.dep[k] = where[r.g][p.dep[k]];
-        p.bulk = (p.kind == PH_FUSED && p.level == 0 && p.ndep == 0) ? 1 : 0;
+        if (p.after >= 0) p.after = where[r.g][p.after];
+        p.bulk = (p.kind == PH_FUSED && p.level == 0 && p.ndep == 0 && p.bulk == 0) ? 1 : 0;
         out.push_back(p);
     }
     // every dependency is an earlier phase and only critical phases have any
-    // (what the kernel's progress guarantee rests on: bulk tasks never wait)
+    // (what the kernel's progress guarantee rests on: bulk tasks never wait);
+    // an IBM starts no earlier than the critical sweep it waits for may
+    for (size_t i = 0; i < out.size(); i++) {
+        const StepPhase& p = out[i];
+        if (p.after < 0) continue;
+        if (p.after >= (int)i || out[p.after].bulk) return false;
+        const StepPhase& w = out[p.after];
+        for (int k = 0; k < w.ndep; k++)
+            if (std::find(p.dep, p.dep + p.ndep, w.dep[k]) == p.dep + p.ndep) return false;
+    }
     for (size_t i = 0; i < out.size(); i++)
         for (int k = 0; k < out[i].ndep; k++) {
             const int d = out[i].dep[k];
@@ -1617,6 +1637,11 @@ sbot_status step_persistent(sbot_ctx* c, int most, int* ran) {
     A.spin_ns = c->spin_ns;
     A.bulk_rounds = c->bulk_rounds;
     A.crit_items = c->crit_items;
+    A.max_servers = c->step_grid / 4;
+    for (int l = 0; l < SBOT_MAXLEV; l++) {
+        const int gl = gl_of(l + 1, l);
+        A.body_count[l] = (((c->groups >> l) & 1) && W_of(c, gl, LK_IBM).cap > 0) ? gl * LK_COUNT + LK_IBM : -1;
+    }
     if (c->prof_mask & 16) {  // the phase trace of this step: [starts (+ launch start)][ends][last starts][first ends][tasks]
         const size_t M = STEP_MAX_PHASES, nst = M + 1;
         if (!c->d_trace) CK(dalloc(&c->d_trace, nst + 3 * M + M / 2));
@@ -1676,7 +1701,7 @@ sbot_status finalize_inst(sbot_ctx* c, int ii) {
     if (I.has_body) {
         const int one[2] = {ii, 1};  // an instance list of one entry, and its length
         TRY(upload(c, c->d_one, one, sizeof one));
-        launch_ibm(c->storage, P, c->d_one, c->d_one + 1, 1, pre_buf(c, fin), fin, 1, I.ibm_smem, c->s);
+        launch_ibm(c->storage, P, c->d_one, c->d_one + 1, 1, pre_buf(c, fin), nullptr, fin, 1, I.ibm_smem, c->s);
         c->launch_n++;
         CK(cudaGetLastError());
     }
@@ -1875,8 +1900,8 @@ sbot_status setup_inst(sbot_ctx* c, int ii, const sbot_domain_desc* desc, const 
     for (int j = 0; j < hb.n; j++) R = std::max(R, std::hypot(hb.qx[j] - hb.pivot[0], hb.qy[j] - hb.pivot[1]));
     int side = (int)std::ceil(2 * R) + 6;
     int cap = side * side;
-    size_t smem = ibm_smem_bytes(c->storage, cap, hb.n);
-    if (smem > ibm_smem_limit(c->storage))
+    const size_t smem = ibm_smem_bytes(c->storage, cap, hb.n);
+    if (ibm_size_bytes(c->storage, cap, hb.n) > ibm_smem_limit(c->storage))
         return fail(c, SBOT_ERR_ARG, "body too large for the one-block IBM kernel");
     I.ibm_smem = smem;
     I.has_body = true;

@@ -40,7 +40,7 @@ namespace {
 template <class S, class C, int COLL, bool SOLID>
 __global__ void __launch_bounds__(1024) k_fused(const __grid_constant__ DevPool P, const int* __restrict__ list, const int* __restrict__ pn,
                                                 const S* __restrict__ fin, S* __restrict__ fout, const S* ffine,
-                                                int level, int allow_force, S* fhalo) {
+                                                int level, S* fhalo) {
     pdl_enter();
     int item = blockIdx.x;
     if (item >= *pn) return;
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(1024) k_fused(const __grid_constant__ DevPool 
     int slot = list[item];
     int cell = threadIdx.x;
     fused_cell<S, C, COLL, SOLID>(P, fin, fout, ffine, slot, P.slot_type[slot], P.inst[P.slot_inst[slot]], level,
-                                  cell % B, cell / B, allow_force != 0, fhalo);
+                                  cell % B, cell / B, fhalo);
 }
 
 // (the LES variants spill at the 80 registers that 3 blocks per SM leave;
@@ -57,13 +57,13 @@ __global__ void __launch_bounds__(1024) k_fused(const __grid_constant__ DevPool 
 template <class S, class C, int B, int COLL>
 __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : 3)
     k_fused_v4(const __grid_constant__ DevPool P, const int* __restrict__ list, const int* __restrict__ pn, const S* __restrict__ fin,
-               S* __restrict__ fout, const S* __restrict__ ffine, int level, int allow_force) {
+               S* __restrict__ fout, const S* __restrict__ ffine, int level) {
     pdl_enter();
     constexpr int SPC = 256 / (B * B / 4);
     const int n = *pn;
     int pass = 0;
     for (int i0 = blockIdx.x * SPC; i0 < n; i0 += gridDim.x * SPC)  // grid stride (vec_grid)
-        fused_v4_task<S, C, B, COLL, true>(P, list, n, i0, pass++, fin, fout, ffine, level, allow_force);
+        fused_v4_task<S, C, B, COLL, true>(P, list, n, i0, pass++, fin, fout, ffine, level);
 }
 
 // Thread blocks of a vector-kernel launch: at most `waves` waves of resident
@@ -91,13 +91,13 @@ unsigned vec_grid(unsigned want, int waves) {
 template <class S, class C, int B, int COLL, bool SH>
 __global__ void __launch_bounds__(256, 3)
     k_fused_v8(const __grid_constant__ DevPool P, const int* __restrict__ list, const int* __restrict__ pn, const S* __restrict__ fin,
-               S* __restrict__ fout, const S* __restrict__ ffine, int level, int allow_force) {
+               S* __restrict__ fout, const S* __restrict__ ffine, int level) {
     pdl_enter();
     constexpr int SPC = 256 / (B * B / 8);
     const int n = *pn;
     int pass = 0;
     for (int i0 = blockIdx.x * SPC; i0 < n; i0 += gridDim.x * SPC)  // grid stride (vec_grid)
-        fused_v8_task<S, C, B, COLL, true, SH>(P, list, n, i0, pass++, fin, fout, ffine, level, allow_force);
+        fused_v8_task<S, C, B, COLL, true, SH>(P, list, n, i0, pass++, fin, fout, ffine, level);
 }
 
 // collision only, on pre-collision populations (the state at t = 0)
@@ -216,7 +216,7 @@ struct TmaSlot {
 template <class S, class C, int B, int COLL>
 __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : (sizeof(S) == 4 ? 3 : 4))
     k_fused_tma(const __grid_constant__ DevPool P, const int* __restrict__ list, const int* __restrict__ pn, const S* __restrict__ fin,
-                S* __restrict__ fout, const S* __restrict__ ffine, int level, int allow_force) {
+                S* __restrict__ fout, const S* __restrict__ ffine, int level) {
     pdl_enter();
     constexpr int BB = B * B, TPS = BB / 4, SPC = 256 / TPS, TPR = B / 4;
     using L = TmaSlot<B>;
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : (sizeof(S) == 4 ? 3 
     const int y = t / TPR, x0 = (t % TPR) * 4;
     if (!fast[ls]) {
         for (int i = 0; i < 4; i++)
-            fused_cell<S, C, COLL, false>(P, fin, fout, ffine, slot, type, ip, level, x0 + i, y, allow_force != 0);
+            fused_cell<S, C, COLL, false>(P, fin, fout, ffine, slot, type, ip, level, x0 + i, y);
         return;
     }
     const S* base = sm + ls * L::elems;
@@ -325,26 +325,12 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : (sizeof(S) == 4 ? 3 
         }
     }
     const C om = (C)1 / (C)ip.tau[level];
-    const int gx0 = P.slot_ox[slot] + x0, gy = P.slot_oy[slot] + y;
-    bool force = false;
-    if (allow_force && ip.has_body && level == ip.m - 1) {  // block meets the IBM force patch?
-        const InstState& st = P.ist[P.slot_inst[slot]];
-        int bx = P.slot_ox[slot], by = P.slot_oy[slot];
-        force = bx < st.patch_x0 + st.patch_w && st.patch_x0 < bx + B && by < st.patch_y0 + st.patch_h &&
-                st.patch_y0 < by + B;
-    }
 #pragma unroll
     for (int i = 0; i < 4; i++) {
         C g[9];
 #pragma unroll
         for (int q = 0; q < 9; q++) g[q] = f[q][i] + dshift<S, C>(ip.dref, q);  // compute form
-        C Fx = 0, Fy = 0;
-        if (force) {
-            patch_force<C>(P, ip, gx0 + i, gy, Fx, Fy);
-            collide_k<COLL, C, true, DevTrait<S>::value, sizeof(S) == 4>(g, om, Fx, Fy, ip);
-        } else {
-            collide_k<COLL, C, false, DevTrait<S>::value, sizeof(S) == 4>(g, om, (C)0, (C)0, ip);
-        }
+        collide_k<COLL, C, false, DevTrait<S>::value, sizeof(S) == 4>(g, om, (C)0, (C)0, ip);
 #pragma unroll
         for (int q = 0; q < 9; q++) f[q][i] = g[q] - dshift<S, C>(ip.dref, q);  // storage form
     }
@@ -370,16 +356,20 @@ __global__ void __launch_bounds__(IBM_THREADS) k_ibm_geom(const __grid_constant_
     ibm_geom_run<C>(P, ilist[item], blockIdx.y, smraw, sh);
 }
 
-template <class S, class C>
+template <class S, class C, int COLL>
 __global__ void __launch_bounds__(IBM_THREADS) k_ibm(const __grid_constant__ DevPool P, const int* __restrict__ ilist,
                                                      const int* __restrict__ pn, const S* __restrict__ fin,
-                                                     int level, int direct, int deferred) {
+                                                     S* __restrict__ fout, int level, int direct, int deferred) {
     pdl_enter();
     const int item = blockIdx.x;
     if (item >= *pn) return;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ IbmShared sh;
-    ibm_run<S, C>(P, ilist[item], fin, level, direct, deferred, smraw, sh, [] { return true; });
+    if (threadIdx.x == 0) sh.geo_inst = -1;
+    __syncthreads();
+    // launched after the sub-step's sweep on the same stream
+    ibm_run<S, C, COLL>(P, ilist[item], fin, fout, level, direct, deferred, -1, smraw, sh, [] { return true; },
+                        [] {}, [] { return true; });
 }
 
 template <class C>
@@ -597,7 +587,7 @@ int storage_bytes(int storage) { return storage == 0 ? 8 : (storage == 1 ? 4 : 2
 
 template <class S, class C, int B, int COLL>
 void launch_tma(const DevPool& P, const int* list, const int* pn, int cap, const void* fin, void* fout,
-                const void* ffine, int level, sbot_stream_t s, int allow_force) {
+                const void* ffine, int level, sbot_stream_t s) {
     constexpr int SPC = 256 / (B * B / 4);
     const size_t smem = (size_t)SPC * TmaSlot<B>::elems * sizeof(S);
     static bool attr_set = false;
@@ -606,16 +596,16 @@ void launch_tma(const DevPool& P, const int* list, const int* pn, int cap, const
         attr_set = true;
     }
     launch_k(P.pdl, k_fused_tma<S, C, B, COLL>, dim3((cap + SPC - 1) / SPC), dim3(256), smem, s, P, list, pn,
-             (const S*)fin, (S*)fout, (const S*)ffine, level, allow_force);
+             (const S*)fin, (S*)fout, (const S*)ffine, level);
 }
 
 template <class S, class C, int COLL>
 void launch_fused_k(const DevPool& P, const int* list, const int* pn, int n, int n_hint, long long vec_min_cells,
                     int staged, const void* fin, void* fout, const void* ffine, int level, sbot_stream_t s,
-                    int allow_force, void* fhalo) {
+                    void* fhalo) {
     if (P.coll & COLL_SOLID) {  // a context holding a solid runs the scalar kernel with the solid links
         launch_k(P.pdl, k_fused<S, C, COLL, true>, dim3(n), dim3(P.B * P.B), 0, s, P, list, pn, (const S*)fin,
-                 (S*)fout, (const S*)ffine, level, allow_force, (S*)fhalo);
+                 (S*)fout, (const S*)ffine, level, (S*)fhalo);
         return;
     }
     // the vector kernel needs enough blocks to fill the GPU: small launches
@@ -623,50 +613,50 @@ void launch_fused_k(const DevPool& P, const int* list, const int* pn, int n, int
     // a launch that also fills the finer level's halo)
     const bool big = fhalo == nullptr && vec_min_cells >= 0 && (long long)n_hint * P.B * P.B >= vec_min_cells;
     if (big && staged && P.B == 16)
-        launch_tma<S, C, 16, COLL>(P, list, pn, n, fin, fout, ffine, level, s, allow_force);
+        launch_tma<S, C, 16, COLL>(P, list, pn, n, fin, fout, ffine, level, s);
     else if (big && staged && P.B == 32)
-        launch_tma<S, C, 32, COLL>(P, list, pn, n, fin, fout, ffine, level, s, allow_force);
+        launch_tma<S, C, 32, COLL>(P, list, pn, n, fin, fout, ffine, level, s);
     else if (big && (P.B == 16 || P.B == 32)) {
         if constexpr (sizeof(S) == 2) {  // 16-bit storage: 8 cells per thread
             const bool sh = (P.coll & COLL_SHIFT) != 0;
             if (P.B == 16)
                 launch_k(P.pdl, sh ? k_fused_v8<S, C, 16, COLL, true> : k_fused_v8<S, C, 16, COLL, false>,
                          dim3(vec_grid((n + 7) / 8, P.vec_waves)), dim3(256), 0, s, P, list, pn, (const S*)fin, (S*)fout, (const S*)ffine,
-                         level, allow_force);
+                         level);
             else
                 launch_k(P.pdl, sh ? k_fused_v8<S, C, 32, COLL, true> : k_fused_v8<S, C, 32, COLL, false>,
                          dim3(vec_grid((n + 1) / 2, P.vec_waves)), dim3(256), 0, s, P, list, pn, (const S*)fin, (S*)fout, (const S*)ffine,
-                         level, allow_force);
+                         level);
         } else {  // FP32 and FP64: 4 cells per thread
             if (P.B == 16)
                 launch_k(P.pdl, k_fused_v4<S, C, 16, COLL>, dim3(vec_grid((n + 3) / 4, P.vec_waves)), dim3(256), 0, s, P, list, pn,
-                         (const S*)fin, (S*)fout, (const S*)ffine, level, allow_force);
+                         (const S*)fin, (S*)fout, (const S*)ffine, level);
             else
                 launch_k(P.pdl, k_fused_v4<S, C, 32, COLL>, dim3(vec_grid(n, P.vec_waves)), dim3(256), 0, s, P, list, pn, (const S*)fin,
-                         (S*)fout, (const S*)ffine, level, allow_force);
+                         (S*)fout, (const S*)ffine, level);
         }
     }
     else
         launch_k(P.pdl, k_fused<S, C, COLL, false>, dim3(n), dim3(P.B * P.B), 0, s, P, list, pn, (const S*)fin,
-                 (S*)fout, (const S*)ffine, level, allow_force, (S*)fhalo);
+                 (S*)fout, (const S*)ffine, level, (S*)fhalo);
 }
 
 void launch_fused(int storage, const DevPool& P, const int* list, const int* pn, int cap, int n_hint,
                   long long vec_min_cells, int staged, const void* fin, void* fout, const void* ffine, int level,
-                  sbot_stream_t s, int allow_force, void* fhalo) {
+                  sbot_stream_t s, void* fhalo) {
     if (cap <= 0) return;
     dispatch(storage, [&](auto* sp, auto* cp) {
         using S = std::remove_pointer_t<decltype(sp)>;
         using C = std::remove_pointer_t<decltype(cp)>;
         if ((P.coll & 15) == 1)
             launch_fused_k<S, C, 1>(P, list, pn, cap, n_hint, vec_min_cells, staged, fin, fout, ffine, level, s,
-                                    allow_force, fhalo);
+                                    fhalo);
         else if ((P.coll & 15) == 2)
             launch_fused_k<S, C, 2>(P, list, pn, cap, n_hint, vec_min_cells, staged, fin, fout, ffine, level, s,
-                                    allow_force, fhalo);
+                                    fhalo);
         else
             launch_fused_k<S, C, 0>(P, list, pn, cap, n_hint, vec_min_cells, staged, fin, fout, ffine, level, s,
-                                    allow_force, fhalo);
+                                    fhalo);
     });
 }
 
@@ -706,7 +696,17 @@ size_t ibm_cache_bytes(int storage, int patch_cap, int n_markers) {
 }
 
 size_t ibm_smem_bytes(int storage, int patch_cap, int n_markers) {
-    // the carve order of k_ibm, each region rounded up to 16 bytes
+    // the carve order of k_ibm, each region rounded up to 16 bytes: the stored
+    // geometry, then the iterations' arrays or the geometry's scratch
+    const size_t c = storage == 0 ? 8 : 4, n = (size_t)n_markers, cap = (size_t)patch_cap;
+    const size_t ncap = cap < 8 * n + 64 ? cap : 8 * n + 64, W = (cap + 31) / 32 + 1;
+    const size_t run = al16(n * c) + 2 * al16(2 * n * c) + 2 * al16(2 * ncap * c) + al16(ncap * c);
+    const size_t scratch = al16(W * 4) + al16((W + 1) * 4) + al16(ncap * 4);
+    return ibm_cache_bytes(storage, patch_cap, n_markers) - sizeof(IbmCacheHead) + (run > scratch ? run : scratch);
+}
+
+size_t ibm_size_bytes(int storage, int patch_cap, int n_markers) {
+    // the size that a body is admitted by: every array in memory of its own
     const size_t c = storage == 0 ? 8 : 4, n = (size_t)n_markers, cap = (size_t)patch_cap;
     const size_t ncap = cap < 8 * n + 64 ? cap : 8 * n + 64, W = (cap + 31) / 32 + 1;
     return ibm_cache_bytes(storage, patch_cap, n_markers) - sizeof(IbmCacheHead) + al16(n * c) + 2 * al16(2 * n * c) +
@@ -724,7 +724,7 @@ size_t ibm_smem_limit(int storage) {
         using S = std::remove_pointer_t<decltype(sp)>;
         using C = std::remove_pointer_t<decltype(cp)>;
         cudaFuncAttributes fa{};
-        stat = cudaFuncGetAttributes(&fa, k_ibm<S, C>) == cudaSuccess ? fa.sharedSizeBytes : 4096;
+        stat = cudaFuncGetAttributes(&fa, k_ibm<S, C, 0>) == cudaSuccess ? fa.sharedSizeBytes : 4096;
     });
     return (size_t)optin > stat ? (size_t)optin - stat : 0;
 }
@@ -758,21 +758,28 @@ void launch_force_sum(int storage, const DevPool& P, const int* inst_list, const
     });
 }
 
-void launch_ibm(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, const void* f,
+template <class S, class C, int COLL>
+void launch_ibm_k(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, const void* f, void* fout,
+                  int level, int direct, size_t smem, sbot_stream_t s, int deferred, int threads) {
+    static bool attr_set = false;
+    if (!attr_set) {
+        cudaFuncSetAttribute(k_ibm<S, C, COLL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)ibm_smem_limit(storage));
+        attr_set = true;
+    }
+    launch_k(P.pdl, k_ibm<S, C, COLL>, dim3(cap), dim3(threads > 0 && threads <= IBM_THREADS ? threads : IBM_THREADS),
+             smem, s, P, inst_list, pn, (const S*)f, (S*)fout, level, direct, deferred);
+}
+
+void launch_ibm(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, const void* f, void* fout,
                 int level, int direct, size_t smem, sbot_stream_t s, int deferred, int threads) {
     if (cap <= 0) return;
-    const int n = cap;
     dispatch(storage, [&](auto* sp, auto* cp) {
         using S = std::remove_pointer_t<decltype(sp)>;
         using C = std::remove_pointer_t<decltype(cp)>;
-        static bool attr_set = false;
-        if (!attr_set) {
-            cudaFuncSetAttribute(k_ibm<S, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)ibm_smem_limit(storage));
-            attr_set = true;
-        }
-        launch_k(P.pdl, k_ibm<S, C>, dim3(n), dim3(threads > 0 && threads <= IBM_THREADS ? threads : IBM_THREADS),
-                 smem, s, P, inst_list, pn, (const S*)f, level, direct, deferred);
+        const int k = P.coll & 15;
+        (k == 1 ? launch_ibm_k<S, C, 1> : (k == 2 ? launch_ibm_k<S, C, 2> : launch_ibm_k<S, C, 0>))(
+            storage, P, inst_list, pn, cap, f, fout, level, direct, smem, s, deferred, threads);
     });
 }
 

@@ -451,8 +451,9 @@ __device__ __forceinline__ void collide9s(C* f, C om, C Fx, C Fy, C cs) {
 
 // the collision of the context's kind: COLL 0 BGK (Eq. 6), 1 MRT, 2 LES.
 // NEQ: the relaxation form of 32-bit storage (bgk_update).
-template <int COLL, class C, bool FORCE, bool DEV, bool NEQ = false>
-__device__ __forceinline__ void collide_k(C* f, C om, C Fx, C Fy, const InstParams& ip) {
+// ip: InstParams, or a copy of its members that are read here.
+template <int COLL, class C, bool FORCE, bool DEV, bool NEQ = false, class IP>
+__device__ __forceinline__ void collide_k(C* f, C om, C Fx, C Fy, const IP& ip) {
     if constexpr (COLL == 1)
         collide9m<C, FORCE, DEV>(f, om, Fx, Fy, (C)ip.mrt_s[0], (C)ip.mrt_s[1], (C)ip.mrt_s[2]);
     else if constexpr (COLL == 2)
@@ -730,15 +731,15 @@ __device__ __forceinline__ void patch_force(const DevPool& P, const InstParams& 
 // ---------------------------------------------------------------------------
 // one cell of the fused step, scalar path: halo cells stream without
 // collision (Sec. 2.4 steps 3, 5); interior cells pull (Eq. 10 + boundary
-// rules), take the IBM force, and collide (Eqs. 3, 6-8)
+// rules) and collide (Eqs. 6-8).  No sweep reads an IBM force: the IBM collides
+// the cells it forces itself (ibm_run), after the sweep has written them.
 // fhalo (non-null): the finer level's buffer whose halo cells inside this
 // level's blocks receive the post-collision populations of the coarse cell
 // that contains them (the coarse-to-fine copy of Sec. 2.4 step 2, done by the
 // cell that owns the values, right after the merge read the same halo cells)
 template <class S, class C, int COLL, bool SOLID, class M>
 __device__ __forceinline__ void fused_cell(const DevPool& P, M mt, const S* fin, S* fout, const S* ffine, int type,
-                                           const InstParams& ip, int level, int x, int y, bool allow_force,
-                                           S* fhalo = nullptr) {
+                                           const InstParams& ip, int level, int x, int y, S* fhalo = nullptr) {
     const int B = P.B, BB = B * B;
     const int cell = y * B + x;
     const int slot = mt.slot();
@@ -770,15 +771,14 @@ __device__ __forceinline__ void fused_cell(const DevPool& P, M mt, const S* fin,
     if constexpr (SOLID) {  // only in contexts holding a solid: the code costs every kernel that contains it
         if ((flags & SLOTF_SOLID) && !solid_links<S, C>(P, fin, slot, ip, level, x, y, f)) return;
     }
-    C Fx = 0, Fy = 0;
-    int gx = mt.ox() + x, gy = mt.oy() + y;
-    if ((flags & SLOTF_EDGE) && inlet_cell<C>(ip, level, gx, gy)) {
+    if ((flags & SLOTF_EDGE) && inlet_cell<C>(ip, level, mt.ox() + x, mt.oy() + y)) {
 #pragma unroll
         for (int q = 0; q < 9; q++) f[q] = feq_s<S, C>(q, (C)ip.rho0, (C)ip.uin_x, (C)ip.uin_y);
-    } else if (allow_force && ip.has_body && level == ip.m - 1) {
-        patch_force<C>(P, ip, gx, gy, Fx, Fy);
     }
-    collide_k<COLL, C, true, DevTrait<S>::value, sizeof(S) == 4>(f, (C)1 / (C)ip.tau[level], Fx, Fy, ip);
+    // (16-bit storage keeps the forced form at zero force: its two forms contract
+    // to different fmas, and one unit of a 16-bit store in every cell's history
+    // is more than a change of schedule may make; the others agree bit for bit)
+    collide_k<COLL, C, sizeof(S) == 2, DevTrait<S>::value, sizeof(S) == 4>(f, (C)1 / (C)ip.tau[level], (C)0, (C)0, ip);
 #pragma unroll
     for (int q = 0; q < 9; q++) Sto<S>::template st<C>(fout, ((size_t)slot * 9 + q) * BB + cell, q, f[q], ip.dref);
     if (fhalo != nullptr && mailbox) {
@@ -801,10 +801,8 @@ __device__ __forceinline__ void fused_cell(const DevPool& P, M mt, const S* fin,
 }
 template <class S, class C, int COLL, bool SOLID>
 __device__ __forceinline__ void fused_cell(const DevPool& P, const S* fin, S* fout, const S* ffine, int slot, int type,
-                                           const InstParams& ip, int level, int x, int y, bool allow_force,
-                                           S* fhalo = nullptr) {
-    fused_cell<S, C, COLL, SOLID, MetaG>(P, MetaG{P, slot}, fin, fout, ffine, type, ip, level, x, y, allow_force,
-                                         fhalo);
+                                           const InstParams& ip, int level, int x, int y, S* fhalo = nullptr) {
+    fused_cell<S, C, COLL, SOLID, MetaG>(P, MetaG{P, slot}, fin, fout, ffine, type, ip, level, x, y, fhalo);
 }
 
 // 4 consecutive values of one population plane, as compute type
@@ -883,7 +881,7 @@ __device__ __forceinline__ uint4 ld_u4(const uint4* p) {
 // read-only path).  Contains a block-wide barrier.
 template <class S, class C, int B, int COLL, bool NC>
 __device__ __forceinline__ void fused_v4_task(const DevPool& P, const int* list, int n, int item0, int pass, const S* fin, S* fout,
-                                              const S* ffine, int level, int allow_force, S* fhalo = nullptr) {
+                                              const S* ffine, int level, S* fhalo = nullptr) {
     static_assert(sizeof(S) >= 4, "16-bit storage takes the 8-cell kernel");
     constexpr int BB = B * B, TPS = BB / 4, TPR = B / 4;
     // two copies: a warp still reading this pass's while another starts the next pass
@@ -900,8 +898,7 @@ __device__ __forceinline__ void fused_v4_task(const DevPool& P, const int* list,
     const int y = t / TPR, x0 = (t % TPR) * 4;
     if (type != ST_INT || (P.slot_flags[slot] & (SLOTF_EDGE | SLOTF_MAILBOX | SLOTF_SOLID))) {
         for (int i = 0; i < 4; i++)
-            fused_cell<S, C, COLL, false>(P, fin, fout, ffine, slot, type, ip, level, x0 + i, y, allow_force != 0,
-                                          fhalo);
+            fused_cell<S, C, COLL, false>(P, fin, fout, ffine, slot, type, ip, level, x0 + i, y, fhalo);
         return;
     }
     C f[9][4];
@@ -972,36 +969,14 @@ __device__ __forceinline__ void fused_v4_task(const DevPool& P, const int* list,
     }
     }
     const C om = (C)1 / (C)ip.tau[level];
-    const int gx0 = P.slot_ox[slot] + x0, gy = P.slot_oy[slot] + y;
-    bool force = false;
-    if (allow_force && ip.has_body && level == ip.m - 1) {  // block meets the IBM force patch?
-        const InstState& st = P.ist[P.slot_inst[slot]];
-        int bx = P.slot_ox[slot], by = P.slot_oy[slot];
-        force = bx < st.patch_x0 + st.patch_w && st.patch_x0 < bx + B && by < st.patch_y0 + st.patch_h &&
-                st.patch_y0 < by + B;
-    }
-    if (force) {
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
-            C g[9];
+    for (int i = 0; i < 4; i++) {
+        C g[9];
 #pragma unroll
-            for (int q = 0; q < 9; q++) g[q] = f[q][i];
-            C Fx = 0, Fy = 0;
-            patch_force<C>(P, ip, gx0 + i, gy, Fx, Fy);
-            collide_k<COLL, C, true, DevTrait<S>::value, sizeof(S) == 4>(g, om, Fx, Fy, ip);
+        for (int q = 0; q < 9; q++) g[q] = f[q][i];
+        collide_k<COLL, C, false, DevTrait<S>::value, sizeof(S) == 4>(g, om, (C)0, (C)0, ip);
 #pragma unroll
-            for (int q = 0; q < 9; q++) f[q][i] = g[q];
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < 4; i++) {
-            C g[9];
-#pragma unroll
-            for (int q = 0; q < 9; q++) g[q] = f[q][i];
-            collide_k<COLL, C, false, DevTrait<S>::value, sizeof(S) == 4>(g, om, (C)0, (C)0, ip);
-#pragma unroll
-            for (int q = 0; q < 9; q++) f[q][i] = g[q];
-        }
+        for (int q = 0; q < 9; q++) f[q][i] = g[q];
     }
 #pragma unroll
     for (int q = 0; q < 9; q++) Vec4<S, C>::st(fout + ((size_t)slot * 9 + q) * BB + y * B + x0, q, f[q]);
@@ -1050,7 +1025,7 @@ __device__ __forceinline__ float el8(const uint4& r, int k) {
 // barrier.
 template <class S, class C, int B, int COLL, bool NC, bool SH>
 __device__ __forceinline__ void fused_v8_task(const DevPool& P, const int* list, int n, int item0, int pass, const S* fin, S* fout,
-                                              const S* ffine, int level, int allow_force, S* fhalo = nullptr) {
+                                              const S* ffine, int level, S* fhalo = nullptr) {
     static_assert(sizeof(S) == 2, "the 8-cell kernel is for 16-bit storage");
     constexpr int BB = B * B, TPS = BB / 8, TPR = B / 8;
     // two copies: a warp still reading this pass's while another starts the next pass
@@ -1067,8 +1042,7 @@ __device__ __forceinline__ void fused_v8_task(const DevPool& P, const int* list,
     const int y = t / TPR, x0 = (t % TPR) * 8;
     if (type != ST_INT || (P.slot_flags[slot] & (SLOTF_EDGE | SLOTF_MAILBOX | SLOTF_SOLID))) {
         for (int i = 0; i < 8; i++)
-            fused_cell<S, C, COLL, false>(P, fin, fout, ffine, slot, type, ip, level, x0 + i, y, allow_force != 0,
-                                          fhalo);
+            fused_cell<S, C, COLL, false>(P, fin, fout, ffine, slot, type, ip, level, x0 + i, y, fhalo);
         return;
     }
     // all nine rows and the edge values requested before any is used
@@ -1101,48 +1075,31 @@ __device__ __forceinline__ void fused_v8_task(const DevPool& P, const int* list,
         }
     }
     const C om = (C)1 / (C)ip.tau[level];
-    const int gx0 = P.slot_ox[slot] + x0, gy = P.slot_oy[slot] + y;
-    bool force = false;
-    if (allow_force && ip.has_body && level == ip.m - 1) {  // block meets the IBM force patch?
-        const InstState& st = P.ist[P.slot_inst[slot]];
-        int bx = P.slot_ox[slot], by = P.slot_oy[slot];
-        force = bx < st.patch_x0 + st.patch_w && st.patch_x0 < bx + B && by < st.patch_y0 + st.patch_h &&
-                st.patch_y0 < by + B;
-    }
     unsigned ow[9][4];
     // SH: values move between the storage and the compute form by the
     // instance's shift (its nine values take registers the kernel is short
     // of, so contexts whose instances all have a zero shift launch SH = false)
     auto shift = [&](int q) { return SH ? (C)ip.dref[q] : (C)0; };
-    auto cells = [&](auto with_force) {
-        constexpr bool F = decltype(with_force)::value;
-        C prev[9];
+    C prev[9];
 #pragma unroll
-        for (int i = 0; i < 8; i++) {
-            C g[9];
+    for (int i = 0; i < 8; i++) {
+        C g[9];
 #pragma unroll
-            for (int q = 0; q < 9; q++) {
-                const int src = i - CXq(q);  // Eq. 10: pull from x - c_q
-                g[q] = (src < 0 || src > 7) ? edge[q] : el8<S>(raw[q], src);
-                if constexpr (SH) g[q] += shift(q);  // compute form
-            }
-            C Fx = 0, Fy = 0;
-            if constexpr (F) patch_force<C>(P, ip, gx0 + i, gy, Fx, Fy);
-            collide_k<COLL, C, F, DevTrait<S>::value, sizeof(S) == 4>(g, om, Fx, Fy, ip);
-#pragma unroll
-            for (int q = 0; q < 9; q++) {
-                const C sq = SH ? g[q] - shift(q) : g[q];  // storage form
-                if (i & 1)
-                    ow[q][i >> 1] = Pair16<S>::pack((float)prev[q], (float)sq);
-                else
-                    prev[q] = sq;
-            }
+        for (int q = 0; q < 9; q++) {
+            const int src = i - CXq(q);  // Eq. 10: pull from x - c_q
+            g[q] = (src < 0 || src > 7) ? edge[q] : el8<S>(raw[q], src);
+            if constexpr (SH) g[q] += shift(q);  // compute form
         }
-    };
-    if (force)
-        cells(std::true_type{});
-    else
-        cells(std::false_type{});
+        collide_k<COLL, C, false, DevTrait<S>::value, sizeof(S) == 4>(g, om, (C)0, (C)0, ip);
+#pragma unroll
+        for (int q = 0; q < 9; q++) {
+            const C sq = SH ? g[q] - shift(q) : g[q];  // storage form
+            if (i & 1)
+                ow[q][i >> 1] = Pair16<S>::pack((float)prev[q], (float)sq);
+            else
+                prev[q] = sq;
+        }
+    }
 #pragma unroll
     for (int q = 0; q < 9; q++)
         *reinterpret_cast<uint4*>(fout + ((size_t)slot * 9 + q) * BB + y * B + x0) =
@@ -1300,12 +1257,21 @@ __device__ void pose_run(const DevPool& P, int inst) {
 // per stencil cell its box index and the start of its marker list; the lists
 // as (marker * 16 + stencil position, kernel weight) records.  Then: per
 // marker the interpolated density, the force and the force increment (pairs);
-// the bitmap with per-word prefix counts; list fill cursors; per stencil cell
-// the velocity being corrected and the force (records of 4), rho and
-// 1/(2 rho).  Records are read and written whole (vector accesses), so each
-// iteration issues about half the shared-memory instructions of one array
-// per component.
+// per stencil cell the velocity being corrected, the force (pairs) and
+// 1/(2 rho).  The geometry's scratch (the bitmap with per-word prefix counts,
+// the list fill cursors) shares the memory of that second part, so that a
+// body of 400 markers fits beside the persistent kernel's own 22 KB.
+//
+// The iterations are bound by shared-memory wavefronts: with the lists read
+// from shared memory in every one, a cell phase of 600 cells issued about
+// 1200 of them (0.6 us).  So each thread keeps its first cell in registers
+// (list, velocity, force, 1/(2 rho), and its populations for the collision),
+// and an iteration reads only the force increments; and the smaller second part
+// lets bodies of up to about 430 markers run in the persistent kernel (the
+// paper's D = 128 cylinder, 402 markers: 456 us per coarse step in the
+// per-phase graphs, 302 there).
 #define IBM_THREADS 1024
+#define IBM_RE 8  // list entries a thread keeps in registers (cells of bodies with markers a cell apart have 3 to 7)
 
 struct IbmCacheHead {  // the first bytes of a stored IBM geometry
     long long stamp;   // moving bodies: the finest time the geometry belongs to
@@ -1339,10 +1305,10 @@ struct IbmSmem {
     size_t cache_bytes;   // the part a stored geometry holds
     C* rj;
     IbmV2<C> *F, *dF;     // [N]
-    unsigned* bits;
+    IbmV2<C> *cu, *cF;    // [ncap]: velocity; force (its x holds rho until the first iteration)
+    C* cinv;              // [ncap]: 1 / (2 rho)
+    unsigned* bits;       // scratch of the geometry, in the memory of the above
     int *wpre, *ccur;
-    IbmV4<C>* cs;         // [ncap]: u x, u y, F x, F y
-    C *crho, *cinv;
 };
 
 template <class C>
@@ -1359,15 +1325,16 @@ __device__ __forceinline__ IbmSmem<C> ibm_carve(unsigned char* smraw, int N, int
     m.cst = carve<int>(sp, ncap + 1);
     m.ent = carve<IbmEnt<C>>(sp, 16LL * N);
     m.cache_bytes = (size_t)(sp - smraw);
+    unsigned char* gp = sp;
     m.rj = carve<C>(sp, N);
     m.F = carve<IbmV2<C>>(sp, N);
     m.dF = carve<IbmV2<C>>(sp, N);
-    m.bits = carve<unsigned>(sp, W);
-    m.wpre = carve<int>(sp, W + 1);
-    m.ccur = carve<int>(sp, ncap);
-    m.cs = carve<IbmV4<C>>(sp, ncap);
-    m.crho = carve<C>(sp, ncap);
+    m.cu = carve<IbmV2<C>>(sp, ncap);
+    m.cF = carve<IbmV2<C>>(sp, ncap);
     m.cinv = carve<C>(sp, ncap);
+    m.bits = carve<unsigned>(gp, W);
+    m.wpre = carve<int>(gp, W + 1);
+    m.ccur = carve<int>(gp, ncap);
     return m;
 }
 
@@ -1468,7 +1435,8 @@ __device__ bool ibm_geometry(const DevPool& P, const InstParams& ip, int level, 
         unsigned b = m.bits[i];
         int r = m.wpre[i];
         while (b) {
-            m.ccell[r++] = i * 32 + (__ffs(b) - 1);
+            const int c = i * 32 + (__ffs(b) - 1);
+            m.ccell[r++] = c % w | (c / w) << 16;
             b &= b - 1;
         }
     }
@@ -1594,7 +1562,20 @@ __device__ void ibm_force_sum(int N, Terms terms, double (*red)[32], double* out
     }
 }
 // the fixed-size shared memory of the IBM and geometry steps
+// A body's parameters, copied before the gate: after it every first read of a
+// global parameter is a round trip to L2 (the acquire of the gate drops the
+// SM's cached lines).
+struct IbmPar {
+    double ds, om;       // Delta s_b, 1 / tau (in FP32 an exact widening)
+    double mrt_s[3], les_cs;
+    int inlet[4], nxl, nyl;
+    float dref[9];
+    int K, fmask;
+    void* fterm;
+};
 struct IbmShared {
+    IbmPar par;
+    int geo_inst;  // the static body whose geometry and parameters this shared memory holds, -1 none
     int bb[4];
     double pose[8];
     double red[3][32];
@@ -1619,6 +1600,7 @@ __device__ void ibm_geom_run(const DevPool& P, int inst, int i, unsigned char* s
     double* const pose = sh.pose;
     int* const wtot = sh.wtot;
     IbmCacheHead& head = sh.head;
+    if (threadIdx.x == 0) sh.geo_inst = -1;
     if (threadIdx.x < 8) pose[threadIdx.x] = ip.pose_tab[4 * i + threadIdx.x];
     __syncthreads();
     IbmCacheHead* e = (IbmCacheHead*)((unsigned char*)ip.ibm_cache + (size_t)i * ip.ibm_cache_stride);
@@ -1628,15 +1610,36 @@ __device__ void ibm_geom_run(const DevPool& P, int inst, int i, unsigned char* s
     }
     ibm_store(e, head, smraw, m.cache_bytes, k0 + i);
 }
+// one direction of a stencil cell's pull without a slot table (a marker box of more than IBM_MAXB blocks a side)
+template <class S, class C>
+__device__ __noinline__ C ibm_pull(const DevPool& P, const S* fin, int slot, const InstParams& ip, int level, int x,
+                                   int y, int q) {
+    return pull_int<S, C>(P, fin, nullptr, false, slot, ip, level, x, y, q);
+}
 // One body's IBM step (k_ibm runs one per thread block); smraw is the
 // block's dynamic shared memory (ibm_smem_bytes), sh its fixed part.
+// direct (the state at t = 0): reads the pre-collision state as it is and
+// leaves the force field in the instance's patch for the first collision.
+// Else it pulls the stencil cells' pre-collision populations from fin, and
+// once it has their force it collides them (Eqs. 3, 6-8) and stores them in
+// fout, over the unforced values this sub-step's sweep wrote there: the sweep
+// then never waits for the IBM, nor the IBM for the sweep until its last
+// stores.  (With the forced blocks swept after the IBM, every finest step was
+// a chain IBM - hand-over - sweep - hand-over.  With the servers of
+// step_impl.cuh, us per coarse step: D = 40 cylinder 63.6 -> 48.7, flapping
+// ellipse 182 -> 148, pitching section 103 -> 82, immersed cylinder in a cavity,
+// 382 markers, 38.7 -> 33.)
+// sub: which finest step of the coarse step this is (-1: not known; the
+// geometry is then looked up by the body's step counter).
 // gate(): called once by the whole block, after the part that may run before
 // the step's earlier phases have finished (the load of a stored geometry)
 // and before the first read of their results; false: stop (the launch is
-// aborting).
-template <class S, class C, class G>
-__device__ void ibm_run(const DevPool& P, int inst, const S* fin, int level, int direct, int deferred,
-                        unsigned char* smraw, IbmShared& sh, G&& gate) {
+// aborting).  await(): called by one whole warp: waits until this sub-step's
+// sweep has finished; swept(), after a barrier that follows it and before the
+// stores to fout: whether it has; false: stop.
+template <class S, class C, int COLL, class G, class G1, class G2>
+__device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int level, int direct, int deferred, int sub,
+                        unsigned char* smraw, IbmShared& sh, G&& gate, G1&& await, G2&& swept) {
     const InstParams& ip = P.inst[inst];
     InstState* st = &P.ist[inst];
     const int B = P.B;
@@ -1652,8 +1655,10 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, int level, int
     double(*const red)[32] = sh.red;
     int* const wtot = sh.wtot;
     IbmCacheHead& head = sh.head;
+    IbmPar& par = sh.par;
 
     const bool still = ip.motion == 0;
+    const bool held = still && sh.geo_inst == inst;  // from this thread block's last IBM
     // the stored geometry of finest step kk, if any: a static body's after
     // its first launch, a moving body's from the geometry step (flag and
     // stamp read with acquire semantics: the entry is complete when seen)
@@ -1666,17 +1671,36 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, int level, int
             (const IbmCacheHead*)((const unsigned char*)ip.ibm_cache + (size_t)i * ip.ibm_cache_stride);
         return ld_acquire_s64(&e->stamp) == kk ? e : nullptr;
     };
+    if (!held) {
+        if (tid == 0) {
+            par.ds = (double)(C)ip.ds;
+            par.om = (double)((C)1 / (C)ip.tau[level]);
+            par.K = ip.K;
+            par.fmask = ip.fterm_n - 1;  // a power of two of entries
+            par.fterm = ip.fterm;
+            par.les_cs = ip.les_cs;
+            for (int i = 0; i < 3; i++) par.mrt_s[i] = ip.mrt_s[i];
+            for (int i = 0; i < 4; i++) par.inlet[i] = ip.bc[i] == BCK_INLET;
+            par.nxl = ip.nx0 << level;
+            par.nyl = ip.ny0 << level;
+        }
+        if (tid < 9) par.dref[tid] = ip.dref[tid];
+    }
     // before the gate: the step counter may still be the previous step's
-    // (its IBM may not have finished); the geometry loaded for it is kept
-    // only if it is the one of the step found after the gate
-    const long long kp = *(volatile const long long*)&st->fine_step;
-    const IbmCacheHead* pre = find_stored(kp);
-    if (pre != nullptr) ibm_load(pre, head, smraw, m.cache_bytes);
+    // (its IBM may not have finished), and so may a moving body's poses; the
+    // geometry loaded here is kept only if it is the one of the step found
+    // after the gate
+    const long long kp = sub >= 0 && !still ? *(volatile const long long*)&st->pose_k0 + sub
+                                            : *(volatile const long long*)&st->fine_step;
+    const IbmCacheHead* pre = held ? (const IbmCacheHead*)ip.ibm_cache : find_stored(kp);
+    if (pre != nullptr && !held) ibm_load(pre, head, smraw, m.cache_bytes);
     if (!gate()) return;
-    const long long k = st->fine_step;
-    const IbmCacheHead* stored = find_stored(k);
+    if (tid == 0 && !held) sh.geo_inst = -1;
+    const long long k = *(volatile const long long*)&st->fine_step;
+    const bool kept = pre != nullptr && (still || k == kp);  // an entry with k's stamp stays k's
+    const IbmCacheHead* stored = kept ? pre : find_stored(k);
     if (stored != nullptr) {
-        if (!(stored == pre && (still || k == kp))) ibm_load(stored, head, smraw, m.cache_bytes);
+        if (!kept) ibm_load(stored, head, smraw, m.cache_bytes);
     } else {
         // pose at t = k and t = k + 1 (Sec. 3.4-3.6): from the coarse step's
         // pose table, else computed here (for motions 1 and 2 with the
@@ -1723,8 +1747,6 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, int level, int
     __syncthreads();
     const int px0 = head.px0, py0 = head.py0, w = head.w, h = head.h, ncell = head.ncell;
     const bool table = head.table != 0;
-    const int pnbx = head.pnbx, pbx0 = head.pbx0, pby0 = head.pby0;
-    const int wh = w * h;
     const int* const ccell = m.ccell;
     const int* const cst = m.cst;
     const IbmEnt<C>* const ent = m.ent;
@@ -1733,73 +1755,103 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, int level, int
     const IbmV4<C>* const mk = m.mk;
     C* const rj = m.rj;
     IbmV2<C>* const dF = m.dF;
-    IbmV4<C>* const cs = m.cs;
-    C* const crho = m.crho;
+    IbmV2<C>* const cu = m.cu;
+    IbmV2<C>* const cF = m.cF;
     C* const cinv = m.cinv;
-    // uncorrected moments of the pre-collision state on the stencil cells (Sec. 2.2 after Eq. 11)
-    for (int ci = tid; ci < ncell; ci += nt) {
-        const int c = ccell[ci];
-        const int gx = px0 + c % w, gy = py0 + c / w;
-        C r = 1, jx = 0, jy = 0;
-        const int bi = table ? (gy / B - pby0) * pnbx + (gx / B - pbx0) : 0;
-        if (table && pslot[bi * 9 + 4] >= 0) {
-            const int x = gx % B, y = gy % B;
-            r = 0;  // deviations: rho = 1 + the sum, the 1 added last (the sum keeps its low bits)
+    const int lb = 31 - __clz(B), BB = B * B, pnbx = head.pnbx, pbx0 = head.pbx0, pby0 = head.pby0;
+    // the pre-collision populations of stencil cell ci (compute form) and the
+    // index of its population 0 (-1: not a finest interior cell with a source
+    // in every direction)
+    auto pull = [&](int ci, C* v) -> long long {
+        const int c = ccell[ci], gx = px0 + (c & 0xffff), gy = py0 + (c >> 16);
+        if (table) {
+            const int* const ps = pslot + 9 * (((gy >> lb) - pby0) * pnbx + (gx >> lb) - pbx0);
+            const int x = gx & (B - 1), y = gy & (B - 1), slot = ps[4];
+            if (slot < 0) return -1;
+            const long long own = (long long)slot * 9 * BB + y * B + x;
             bool ok = true;
 #pragma unroll
             for (int q = 0; q < 9; q++) {
-                C v;
                 if (direct) {
-                    v = Sto<S>::template ld<C>(fin, ((size_t)pslot[bi * 9 + 4] * 9 + q) * B * B + y * B + x, q,
-                                               ip.dref);
-                } else {
-                    const int sx = x - CXq(q), sy = y - CYq(q);
-                    const int dx = sx < 0 ? -1 : (sx >= B ? 1 : 0), dy = sy < 0 ? -1 : (sy >= B ? 1 : 0);
-                    const int ns = pslot[bi * 9 + (dy + 1) * 3 + dx + 1];
-                    ok &= ns >= 0;
-                    v = ns >= 0 ? Sto<S>::template ld<C>(
-                                      fin, ((size_t)ns * 9 + q) * B * B + (sy - dy * B) * B + (sx - dx * B), q,
-                                      ip.dref)
-                                : (C)0;
+                    v[q] = Sto<S>::template ld<C>(fin, own + q * BB, q, par.dref);
+                    continue;
                 }
-                r += v;
-                jx += (C)CXq(q) * v;
-                jy += (C)CYq(q) * v;
+                const int sx = x - CXq(q), sy = y - CYq(q);
+                const int dx = sx < 0 ? -1 : (sx >= B ? 1 : 0), dy = sy < 0 ? -1 : (sy >= B ? 1 : 0);
+                const int ns = ps[(dy + 1) * 3 + dx + 1];
+                ok &= ns >= 0;
+                v[q] = Sto<S>::template ld<C>(
+                    fin, ((size_t)max(ns, 0) * 9 + q) * BB + (sy & (B - 1)) * B + (sx & (B - 1)), q, par.dref);
+            }
+            return ok ? own : -1;
+        }
+        const int slot = lat_slot(P, ip, level, gx, gy);
+        if (slot < 0 || P.slot_type[slot] != ST_INT) return -1;
+        const int x = gx - P.slot_ox[slot], y = gy - P.slot_oy[slot];
+        const long long own = (long long)slot * 9 * BB + y * B + x;
+#pragma unroll
+        for (int q = 0; q < 9; q++)
+            v[q] = direct ? Sto<S>::template ld<C>(fin, own + q * BB, q, ip.dref)
+                          : ibm_pull<S, C>(P, fin, slot, ip, level, x, y, q);
+        return own;
+    };
+    // uncorrected moments of the pre-collision state on the stencil cells (Sec. 2.2 after Eq. 11)
+    auto moments = [&](int ci, C* v, IbmV2<C>& u, C& inv) -> long long {
+        C r = 1, jx = 0, jy = 0;
+        const long long own = pull(ci, v);
+        if (own >= 0) {
+            r = 0;  // deviations: rho = 1 + the sum, the 1 added last (the sum keeps its low bits)
+#pragma unroll
+            for (int q = 0; q < 9; q++) {
+                r += v[q];
+                jx += (C)CXq(q) * v[q];
+                jy += (C)CYq(q) * v[q];
             }
             if (DevTrait<S>::value) r += (C)1;
-            if (!ok) {
-                atomicOr(P.err, ERRB_STENCIL);
-                r = 1;
-            }
-        } else if (!table) {
-            const int slot = lat_slot(P, ip, level, gx, gy);
-            if (slot < 0 || P.slot_type[slot] != ST_INT) {
-                atomicOr(P.err, ERRB_STENCIL);
-            } else {
-                const int x = gx - P.slot_ox[slot], y = gy - P.slot_oy[slot];
-                r = 0;
-#pragma unroll
-                for (int q = 0; q < 9; q++) {
-                    C v = direct ? Sto<S>::template ld<C>(fin, ((size_t)slot * 9 + q) * B * B + y * B + x, q, ip.dref)
-                                 : pull_int<S, C>(P, fin, nullptr, false, slot, ip, level, x, y, q);
-                    r += v;
-                    jx += (C)CXq(q) * v;
-                    jy += (C)CYq(q) * v;
-                }
-                if (DevTrait<S>::value) r += (C)1;
-            }
         } else {
             atomicOr(P.err, ERRB_STENCIL);
         }
-        crho[ci] = r;
-        cinv[ci] = (C)1 / ((C)2 * r);
-        cs[ci] = IbmV4<C>{jx / r, jy / r, (C)0, (C)0};
+        inv = (C)1 / ((C)2 * r);
+        u = IbmV2<C>{jx / r, jy / r};
+        cu[ci] = u;
+        cF[ci].x = r;
+        return own;
+    };
+    // this thread's first cell: its populations, velocity, force, and the
+    // first IBM_RE entries of its list (marker and weight)
+    C f0[9], inv0 = 0, ew[IBM_RE];
+    IbmV2<C> u0{}, F0{(C)0, (C)0};
+    unsigned em[IBM_RE / 2];
+    int e0 = 0, e1 = 0;
+    long long own0 = -1;
+#pragma unroll
+    for (int i = 0; i < IBM_RE; i++) ew[i] = 0;
+#pragma unroll
+    for (int i = 0; i < IBM_RE / 2; i++) em[i] = 0;
+    if (tid < ncell) {
+        own0 = moments(tid, f0, u0, inv0);
+        e0 = cst[tid];
+        e1 = cst[tid + 1];
+#pragma unroll
+        for (int i = 0; i < IBM_RE; i++) {
+            if (e0 + i < e1) {
+                const IbmEnt<C> en = ent[e0 + i];
+                em[i >> 1] |= (unsigned)(en.m16 >> 4) << (16 * (i & 1));
+                ew[i] = en.w;
+            }
+        }
+    }
+    for (int ci = tid + nt; ci < ncell; ci += nt) {
+        C v[9], inv;
+        IbmV2<C> u;
+        moments(ci, v, u, inv);
+        cinv[ci] = inv;
     }
     __syncthreads();
-    const C ds = (C)ip.ds;
+    const C ds = (C)par.ds;
     // K iterations: per marker Eq. 12 over its 16 cells and Eq. 11; per cell
     // Eq. 15 over its markers and the correction of Eq. 8
-    const int K = ip.K;
+    const int K = par.K;
     for (int it = 0; it < K; it++) {
         for (int j = tid; j < N; j += nt) {
             C u = 0, v = 0, r = 0;
@@ -1811,10 +1863,10 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, int level, int
             for (int s16 = 0; s16 < 16; s16++) {
                 const int ci = (iw[s16 >> 1] >> (16 * (s16 & 1))) & 0xffffu;
                 const C d = wxa[s16 & 3] * wya[s16 >> 2];
-                const IbmV2<C> cu = *(const IbmV2<C>*)(cs + ci);
-                u += cu.x * d;
-                v += cu.y * d;
-                if (it == 0) r += crho[ci] * d;
+                const IbmV2<C> uc = cu[ci];
+                u += uc.x * d;
+                v += uc.y * d;
+                if (it == 0) r += cF[ci].x * d;
             }
             if (it == 0) rj[j] = r;
             const C rr = it == 0 ? r : rj[j];
@@ -1828,7 +1880,36 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, int level, int
             F[j] = fj;
         }
         __syncthreads();
-        for (int ci = tid; ci < ncell; ci += nt) {
+        if (tid < ncell) {
+            C sx = 0, sy = 0;
+#pragma unroll
+            for (int h = 0; h < IBM_RE; h += 4) {
+                if (e0 + h >= e1) break;
+                IbmV2<C> d[4];
+#pragma unroll
+                for (int i = 0; i < 4; i++)  // past the list's end: marker 0 with weight 0, not read
+                    d[i] = e0 + h + i < e1 ? dF[(em[(h + i) >> 1] >> (16 * (i & 1))) & 0xffffu] : IbmV2<C>{(C)0, (C)0};
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    sx += ew[h + i] * d[i].x;
+                    sy += ew[h + i] * d[i].y;
+                }
+            }
+            for (int e = e0 + IBM_RE; e < e1; e++) {
+                const IbmEnt<C> en = ent[e];
+                const IbmV2<C> d = dF[en.m16 >> 4];
+                sx += en.w * d.x;
+                sy += en.w * d.y;
+            }
+            sx *= ds;  // Eq. 15
+            sy *= ds;
+            F0.x += sx;
+            F0.y += sy;
+            u0.x += sx * inv0;
+            u0.y += sy * inv0;
+            cu[tid] = u0;
+        }
+        for (int ci = tid + nt; ci < ncell; ci += nt) {
             C sx = 0, sy = 0;
             const int b1 = cst[ci + 1];
             for (int e = cst[ci]; e < b1; e++) {
@@ -1837,33 +1918,33 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, int level, int
                 sx += en.w * d.x;
                 sy += en.w * d.y;
             }
-            sx *= ds;  // Eq. 15
+            sx *= ds;
             sy *= ds;
-            IbmV4<C> c = cs[ci];
+            IbmV2<C> c = cu[ci], g = it == 0 ? IbmV2<C>{(C)0, (C)0} : cF[ci];
             const C iv = cinv[ci];
-            c.z += sx;
-            c.w += sy;
+            g.x += sx;
+            g.y += sy;
             c.x += sx * iv;
             c.y += sy * iv;
-            cs[ci] = c;
+            cF[ci] = g;
+            cu[ci] = c;
         }
         __syncthreads();
     }
-    // the force field: zero on the box, the accumulated force on the stencil
-    // cells (a static body with a stored geometry writes the same cells as the
-    // launch that stored it, whose zeros the rest of the box still holds)
-    C* gF = (C*)ip.patch;
-    if (!(still && stored != nullptr)) {
-        for (int c = tid; c < wh; c += nt) {
+    if (direct) {
+        // the force field: zero on the box, the accumulated force on the stencil cells
+        C* gF = (C*)ip.patch;
+        for (int c = tid; c < w * h; c += nt) {
             gF[c] = 0;
             gF[cap + c] = 0;
         }
         __syncthreads();
-    }
-    for (int ci = tid; ci < ncell; ci += nt) {
-        const int c = ccell[ci];
-        gF[c] = cs[ci].z;
-        gF[cap + c] = cs[ci].w;
+        for (int ci = tid; ci < ncell; ci += nt) {
+            const int c = (ccell[ci] >> 16) * w + (ccell[ci] & 0xffff);
+            const IbmV2<C> g = ci == tid ? F0 : cF[ci];
+            gF[c] = g.x;
+            gF[cap + c] = g.y;
+        }
     }
     // a static body keeps its geometry for the next launches
     if (still && ip.ibm_cache != nullptr && stored == nullptr)
@@ -1881,7 +1962,7 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, int level, int
     };
     const bool store_cache = still && ip.ibm_cache != nullptr && stored == nullptr;
     if (deferred) {
-        C* out = (C*)ip.fterm + (size_t)(k % ip.fterm_n) * 3 * N;
+        C* out = (C*)par.fterm + (size_t)(k & par.fmask) * 3 * N;
         for (int j = tid; j < N; j += nt) {
             C a, b, mm;
             terms(j, a, b, mm);
@@ -1893,7 +1974,35 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, int level, int
     } else {
         ibm_force_sum<C>(N, terms, red, ip.hist + 3 * (k % SBOT_HIST_CAP));
     }
+    if (!direct) {
+        // the forced collision of the stencil cells (an inlet cell keeps the
+        // sweep's value: it is reset to the inlet state after streaming)
+        const C om = (C)par.om;
+        if (wid == (nt >> 5) - 1) await();  // often a warp without cells
+        for (int ci = tid, r = 0; r == 0 || ci < ncell; ci += nt, r++) {
+            if (r > 0) own0 = pull(ci, f0);
+            bool ok = own0 >= 0;
+            if (ok) {
+                const int c = ccell[ci], gx = px0 + (c & 0xffff), gy = py0 + (c >> 16);
+                ok = !((gx == 0 && par.inlet[SIDE_W]) || (gx == par.nxl - 1 && par.inlet[SIDE_E]) ||
+                       (gy == 0 && par.inlet[SIDE_S]) || (gy == par.nyl - 1 && par.inlet[SIDE_N]));
+            }
+            if (ok) {
+                if (r > 0) F0 = cF[ci];
+                collide_k<COLL, C, true, DevTrait<S>::value, sizeof(S) == 4>(f0, om, F0.x, F0.y, par);
+            }
+            if (r == 0) {  // by now the sweep has mostly finished
+                __syncthreads();
+                if (!swept()) return;
+            }
+            if (ok) {
+#pragma unroll
+                for (int q = 0; q < 9; q++) Sto<S>::template st<C>(fout, own0 + q * BB, q, f0[q], par.dref);
+            }
+        }
+    }
     if (tid == 0) {
+        sh.geo_inst = still && stored != nullptr ? inst : -1;
         st->patch_x0 = px0;
         st->patch_y0 = py0;
         st->patch_w = w;

@@ -137,8 +137,6 @@ constexpr int COLL_SHIFT = 32;
 // A launch of n_hint blocks of at least vec_min_cells cells takes the vector
 // kernel (4 cells per thread, 8 in 16-bit storage; B = 16 or 32), a smaller one the scalar kernel
 // (one cell per thread); vec_min_cells < 0 never takes the vector kernel.
-// allow_force = 0: the launch reads no IBM force (blocks known to lie outside
-// every patch).
 // ffine: the next finer level's buffer after its two sub-steps (read by the
 // merge of populations streaming in from the finer region; unused on levels
 // without a finer one).
@@ -150,7 +148,7 @@ constexpr int COLL_SHIFT = 32;
 // sub-step); such a launch takes the one-cell-per-thread kernel.
 void launch_fused(int storage, const DevPool& P, const int* list, const int* pn, int cap, int n_hint,
                   long long vec_min_cells, int staged, const void* fin, void* fout, const void* ffine, int level,
-                  sbot_stream_t s, int allow_force = 1, void* fhalo = nullptr);
+                  sbot_stream_t s, void* fhalo = nullptr);
 void launch_collide_init(int storage, const DevPool& P, const int* list, int n, const void* fpre, void* fpost,
                          int level, sbot_stream_t s);
 void launch_c2f(int storage, const DevPool& P, const int* list, const int* pn, int cap, const void* fcoarse,
@@ -161,13 +159,16 @@ void launch_pose(const DevPool& P, const int* inst_list, const int* pn, int cap,
 // for launch_force_sum, which sums the `steps` finest steps of the coarse
 // step just run
 // threads: the thread block that runs one body (at most 1024)
+// direct = 0: collides the cells it forces and stores them in fout, over what
+// the sub-step's sweep (launched before it on the same stream) wrote there
 void launch_ibm(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, const void* f,
-                int level, int direct, size_t smem, sbot_stream_t s, int deferred = 0, int threads = 1024);
+                void* fout, int level, int direct, size_t smem, sbot_stream_t s, int deferred = 0, int threads = 1024);
 void launch_force_sum(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, int steps,
                       sbot_stream_t s);
 void launch_ibm_geom(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, int steps,
                      size_t smem, sbot_stream_t s);
 size_t ibm_smem_bytes(int storage, int patch_cap, int n_markers);
+size_t ibm_size_bytes(int storage, int patch_cap, int n_markers);  // at least that: what the admission limit counts
 size_t ibm_smem_limit(int storage);  // largest dynamic shared memory k_ibm can launch with
 size_t ibm_cache_bytes(int storage, int patch_cap, int n_markers);
 void launch_export(int storage, const DevPool& P, const int* list, int n, const void* f, const void* ffine, int level,
@@ -209,12 +210,12 @@ struct StepPhase {
     int kind;         // PH_*
     int bulk;         // 1: bulk queue (no dependencies); 0: critical queue
     int level;
-    int allow_force;  // PH_FUSED: 0 when no block of the list meets a force patch
+    int after;        // PH_IBM: the sweep of its sub-step (an earlier phase), awaited before its stores; else -1
     int fin, fout, ffine;  // population buffers by index (0, 1), -1 none
     int list_off;     // the work list: offset in the device list array
     int count_idx;    // its length: index in the device count array
     int fold;         // PH_FUSED: its cells next to the finer region also write the finer level's halo (in ffine)
-    int arg;          // PH_GEOM: finest step of the coarse step; PH_FSUM: finest steps per coarse step;
+    int arg;          // PH_GEOM, PH_IBM: finest step of the coarse step; PH_FSUM: finest steps per coarse step;
                       // PH_FUSED: 1 to keep one cell per thread (blocks whose pulls merge fine values)
     int ndep;
     int dep[STEP_MAX_DEPS];   // the phases this one waits for (all earlier; a bulk phase waits for none)
@@ -242,6 +243,8 @@ struct StepArgs {
     long long spin_ns;        // longest wait for a dependency before the launch gives up (ERRB_TIMEOUT)
     int bulk_rounds;          // vector rounds per bulk task
     int crit_items;           // > 0: at most this many list items per task of a critical fused phase
+    int max_servers;          // most thread blocks set apart for one body's IBM each (more bodies: no block is)
+    int body_count[SBOT_MAXLEV];  // per group, the index of its body list's length, -1 none
     // phase trace (nullptr: off): device ns of each phase's first task start
     // and last task end, its task count, and the launch's first start
     // (start[STEP_MAX_PHASES])

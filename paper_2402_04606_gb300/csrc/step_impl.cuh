@@ -72,6 +72,9 @@ __device__ __forceinline__ int fused_items(bool vec, int T) {
     return vec ? T / (B * B / CPT) : (T >= B * B ? T / (B * B) : 1);
 }
 
+// the most list items whose blocks' data a task of a sweep reads ahead
+#define STEP_META_MAX (STEP_MAX_THREADS / 64)
+
 // How fused phase ph with n items is cut into tasks: `per` items per round and
 // `rounds` rounds per task, or (parts > 1) every item into `parts` tasks of its
 // own.  Handing out a task costs some microseconds of dependent L2 round
@@ -103,8 +106,13 @@ __device__ __forceinline__ TaskShape task_shape(const StepArgs& A, const StepPha
     if (ph.bulk || n > 8 * fill) {
         const long long waves = (n + fill * A.bulk_rounds - 1) / (fill * A.bulk_rounds);
         t.rounds = (int)((n + fill * waves - 1) / (fill * waves));
-    } else if (A.crit_items > 0 && A.crit_items < t.per) {
-        t.per = A.crit_items;
+    } else if (A.crit_items > 0) {
+        t.per = min(t.per, A.crit_items);
+    } else if (!vec && n > fill) {
+        // a critical sweep of more fillings than one: a single task per thread
+        // block where its blocks' data fit (STEP_META_MAX)
+        const int want = (int)((n + fill - 1) / fill) * t.per;
+        t.per = min(want, min(STEP_META_MAX, T / 32) / t.per * t.per);
     }
     if (sizeof(S) == 8 && n < fill) t.per = (n + grid - 1) / grid;
     if (sizeof(S) == 8 && !vec && 2LL * n <= grid) t.parts = 4LL * n <= grid ? 4 : 2;
@@ -140,10 +148,6 @@ __device__ __forceinline__ void for_cells(int n, int i0, int k, int BB, F&& fn) 
     }
 }
 
-// the most list items a scalar task of a critical sweep holds (T / (B * B)
-// for B >= 8)
-#define STEP_META_MAX (STEP_MAX_THREADS / 64)
-
 // A fused phase's task.  gate(): see step_task.  A critical task on the
 // scalar mapping first reads its blocks' data (slot tables, neighbours and
 // their types, children) into shared memory, which it may do before the
@@ -173,7 +177,7 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
             const SlotMeta& m = meta[c / (B * B)];
             const int cell = c % (B * B);
             fused_cell<S, C, COLL, false, MetaS>(P, MetaS{&m}, fin, fout, ffine, m.type, P.inst[m.inst], ph.level,
-                                                 cell % B, cell / B, ph.allow_force != 0, fhalo);
+                                                 cell % B, cell / B, fhalo);
         }
         return;
     }
@@ -186,17 +190,16 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
             if (vec) {
                 if constexpr (sizeof(S) == 2)
                     fused_v8_task<S, C, B, COLL, false, true>(P, list, ne, i0, r, fin, fout, ffine, ph.level,
-                                                              ph.allow_force, fhalo);
+                                                              fhalo);
                 else
-                    fused_v4_task<S, C, B, COLL, false>(P, list, ne, i0, r, fin, fout, ffine, ph.level, ph.allow_force,
-                                                        fhalo);
+                    fused_v4_task<S, C, B, COLL, false>(P, list, ne, i0, r, fin, fout, ffine, ph.level, fhalo);
                 continue;
             }
         }
         for_cells(ne, i0, per, B * B, [&](int item, int cell) {
             const int slot = list[item];
             fused_cell<S, C, COLL, false>(P, fin, fout, ffine, slot, P.slot_type[slot], P.inst[P.slot_inst[slot]],
-                                          ph.level, cell % B, cell / B, ph.allow_force != 0, fhalo);
+                                          ph.level, cell % B, cell / B, fhalo);
         });
     }
 }
@@ -207,9 +210,11 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
 // before it.  prologue: the task wrote shared memory before it (a barrier
 // is then due even when there is nothing to wait for).  It returns false
 // when the launch is aborting (the task then stops).
-template <class S, class C, int B, int COLL, class G>
+// An IBM task waits before its stores for the sweep of its sub-step
+// (ph.after): await() by one warp, swept() by all after a barrier (ibm_run).
+template <class S, class C, int B, int COLL, class G, class G1, class G2>
 __device__ void step_task(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, unsigned char* smraw,
-                          IbmShared& sh, G& gate) {
+                          IbmShared& sh, G& gate, G1& await, G2& swept) {
     const int* list = A.lists + ph.list_off;
     if (A.counts[ph.count_idx] <= 0) {  // the empty task of a phase with no work
         gate(false);
@@ -217,7 +222,10 @@ __device__ void step_task(const DevPool& P, const StepArgs& A, const StepPhase& 
     }
     switch (ph.kind) {
     case PH_FUSED: step_fused<S, C, B, COLL>(P, A, ph, local, gate); break;
-    case PH_IBM: ibm_run<S, C>(P, list[local], step_buf<S>(A, ph.fin), ph.level, 0, 1, smraw, sh, gate); break;
+    case PH_IBM:
+        ibm_run<S, C, COLL>(P, list[local], step_buf<S>(A, ph.fin), step_buf<S>(A, ph.fout), ph.level, 0, 1, ph.arg,
+                            smraw, sh, gate, await, swept);
+        break;
     default: {
         if (!gate(false)) return;
         switch (ph.kind) {
@@ -309,13 +317,14 @@ __device__ __forceinline__ bool deps_acquire(const StepArgs& A, const StepDeps& 
     return __all_sync(0xffffffffu, ok);
 }
 
-// Warp 0, all lanes: wait until every dependency of phase q has finished,
-// bounded by A.spin_ns of device time; false when the launch is aborting (by
-// this wait or another)
-__device__ bool wait_deps(const DevPool& P, const StepArgs& A, const StepDeps& D, int q, const int* ntask) {
+// Warp 0, all lanes: wait until ready() (acquire loads, the same answer in
+// every lane), bounded by A.spin_ns of device time; false when the launch is
+// aborting (by this wait or another)
+template <class R>
+__device__ bool wait_until(const DevPool& P, const StepArgs& A, R&& ready) {
     const unsigned long long t0 = global_ns();
     for (unsigned ns = 16;; ns = ns < 64 ? 2 * ns : ns) {  // short naps: each poll is an L2 round trip anyway
-        if (deps_acquire(A, D, q, ntask)) return true;
+        if (ready()) return true;
         int stop = 0;
         if ((threadIdx.x & 31) == 0) {
             if (ld_relaxed(&A.ctl->abort)) {
@@ -342,11 +351,33 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
     __shared__ int wtot[32];
     // the scheduler's state lives in shared memory, so that no register is
     // held across a task (the vector sweep needs all of them)
-    __shared__ int s_cmd, s_phase, s_local, s_last, s_ncp, s_nbulk, s_bulk_left;
+    __shared__ int s_cmd, s_phase, s_local, s_last, s_ncp, s_nbulk, s_bulk_left, s_turn;
     __shared__ int s_wait, s_go;  // the claimed critical phase to wait for (-1: none), the wait's outcome
+    __shared__ int s_body[SBOT_MAXLEV + 1];  // first server of each group's bodies, their number
     const int tid = threadIdx.x, nph = A.nph;
     StepCtl* ctl = A.ctl;
     constexpr unsigned FULL = 0xffffffffu;
+
+    // IBM servers: where there are at most max_servers bodies, the first
+    // thread blocks run one body's IBM each and nothing else, so that the IBM's
+    // code and its data stay in that SM's caches, a static body's geometry in
+    // its shared memory, and one step's IBM follows the last without a
+    // hand-over between SMs (D = 40 cylinder 54.7 -> 50.2 us per coarse step, the
+    // D = 128 one 361 against 453 with the IBM handed out after the sweep's tasks)
+    if (tid == 0) {
+        int n = 0;
+        for (int g = 0; g < SBOT_MAXLEV; g++) {
+            s_body[g] = n;
+            if (A.body_count[g] >= 0) n += max(A.counts[A.body_count[g]], 0);
+        }
+        s_body[SBOT_MAXLEV] = n <= A.max_servers ? n : 0;
+        s_turn = 0;
+        sh.geo_inst = -1;
+    }
+    __syncthreads();
+    const int nsrv = s_body[SBOT_MAXLEV];
+    const bool server = (int)blockIdx.x < nsrv;
+    auto served = [&](const StepPhase& ph) { return nsrv > 0 && ph.kind == PH_IBM && A.counts[ph.count_idx] > 0; };
 
     // task counts from this launch's list lengths (a critical phase with no
     // work but with dependencies gets one empty task, so that the phases after
@@ -359,7 +390,7 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
         ntask[p] = nt;
         deps.n[p] = ph.ndep;
         for (int k = 0; k < ph.ndep; k++) deps.d[p][k] = (unsigned short)ph.dep[k];
-        cpos[p] = (!ph.bulk && nt > 0) ? 1 : 0;
+        cpos[p] = (!ph.bulk && nt > 0 && served(ph) == server) ? 1 : 0;
         bfirst[p] = ph.bulk ? nt : 0;
     }
     __syncthreads();
@@ -372,13 +403,28 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
             s_bulk_left = nbulk > 0;
         }
     }
-    for (int p = tid; p < nph; p += blockDim.x)
-        if (!A.ph[p].bulk && ntask[p] > 0) crit[cpos[p]] = p;
+    for (int p = tid; p < nph; p += blockDim.x) {
+        const StepPhase& ph = A.ph[p];
+        if (!ph.bulk && ntask[p] > 0 && served(ph) == server) crit[cpos[p]] = p;
+    }
     __syncthreads();
     if (A.tr_start && tid == 0) atomicMin(&A.tr_start[STEP_MAX_PHASES], global_ns());
 
     for (;;) {
-        if (threadIdx.x < 32) {  // warp 0 decides
+        if (server) {
+            if (threadIdx.x == 0) {  // the next IBM phase that its body has
+                int i = s_turn, local = 0;
+                for (; i < s_ncp; i++) {
+                    local = (int)blockIdx.x - s_body[A.ph[crit[i]].level];  // (a body's group is its finest level)
+                    if (local >= 0 && local < ntask[crit[i]]) break;
+                }
+                s_turn = i + 1;
+                s_cmd = i < s_ncp ? STEP_RUN : STEP_EXIT;
+                s_phase = s_wait = i < s_ncp ? crit[i] : -1;
+                s_local = local;
+                s_go = 1;
+            }
+        } else if (threadIdx.x < 32) {  // warp 0 decides
             const int lane = threadIdx.x, ncp = s_ncp, nbulk = s_nbulk;
             int cmd = STEP_EXIT, p = -1, local = 0;
             int wq = -1;  // a claimed critical phase: its dependencies are read with acquire before it runs
@@ -474,7 +520,7 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
             __syncthreads();
             if (threadIdx.x < 32) {
                 const int q = s_wait;
-                const bool ok = q < 0 || wait_deps(P, A, deps, q, ntask);
+                const bool ok = q < 0 || wait_until(P, A, [&] { return deps_acquire(A, deps, q, ntask); });
                 if (threadIdx.x == 0) {
                     s_go = ok;
                     if (ok && A.tr_start) {
@@ -487,7 +533,17 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
             __syncthreads();
             return s_go != 0;
         };
-        step_task<S, C, B, COLL>(P, A, A.ph[s_phase], s_local, smraw, sh, gate);
+        // an IBM task before its stores: the sweep of its sub-step has
+        // finished (no deadlock: that phase is ready whenever the IBM is, and
+        // earlier in the order, so all its tasks were taken before this one,
+        // and a sweep's task never waits after its gate)
+        auto await = [&]() {
+            const int d = A.ph[s_phase].after;
+            const bool ok = d < 0 || wait_until(P, A, [&] { return ld_acquire(&A.ctl->done[d]) >= ntask[d]; });
+            if ((threadIdx.x & 31) == 0 && !ok) s_go = 0;
+        };
+        auto swept = [&]() -> bool { return s_go != 0; };
+        step_task<S, C, B, COLL>(P, A, A.ph[s_phase], s_local, smraw, sh, gate, await, swept);
         __syncthreads();  // the task's writes, then its count (a release: the
                           // barrier orders every thread's writes before it)
         if (threadIdx.x == 0 && s_go) {
@@ -500,6 +556,7 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
             }
             red_release_add(&ctl->done[p], 1);
         }
+        if (server && !s_go) break;
     }
     // the last thread block to leave zeroes the control block for the next launch
     if (threadIdx.x == 0) {

@@ -109,6 +109,7 @@ struct Inst {
     double* d_pose = nullptr;
     void* d_ibmcache = nullptr;
     void* d_fterm = nullptr;
+    void* d_solid = nullptr;
     long long coarse_step = 0;  // this instance's own time
     long long forces_read = 0;
     bool finalized = false;
@@ -1071,6 +1072,7 @@ sbot_status build_topology(sbot_ctx* c, int ii, long long n, bool transfer) {
         }
     }
     std::vector<int> ints;
+    I.ip.solid_blocks = 0;
     for (int l = 0; l < I.m; l++) {
         I.int_off[l] = (int)ints.size();
         for (size_t i = 0; i < planned.size(); i++) {
@@ -1086,8 +1088,10 @@ sbot_status build_topology(sbot_ctx* c, int ii, long long n, bool transfer) {
                     if (nb >= 0 && c->h_type[nb] == ST_GC) dep = true;
                 }
                 if (dep) set_tab(c, c->h_flags, A_FLAGS, sl, c->h_flags[sl] | (int)SLOTF_MAILBOX);
-                if (l == I.m - 1 && solid_near_block(I.ip, pb.bx * c->B, pb.by * c->B, c->B))
+                if (l == I.m - 1 && solid_near_block(I.ip, pb.bx * c->B, pb.by * c->B, c->B)) {
                     set_tab(c, c->h_flags, A_FLAGS, sl, c->h_flags[sl] | (int)SLOTF_SOLID);
+                    set_tab(c, c->h_parent, A_PARENT, sl, I.ip.solid_blocks++);  // its entry in the links' table
+                }
                 if (l == I.m - 1 && I.has_body) {
                     int x0 = pb.bx * c->B, y0 = pb.by * c->B;
                     dep = dep || !static_body || (x0 <= bx1 && bx0 < x0 + c->B && y0 <= by1 && by0 < y0 + c->B);
@@ -1110,6 +1114,14 @@ sbot_status build_topology(sbot_ctx* c, int ii, long long n, bool transfer) {
         I.int_cap = ncap;
     }
     TRY(upload(c, I.d_int, ints.data(), ints.size() * sizeof(int)));
+    if (I.ip.solid_blocks > 0) {  // the links' table (filled once the slot tables are written, by admit)
+        CK(cudaStreamSynchronize(c->s));
+        dfree(I.d_solid);
+        I.d_solid = nullptr;
+        CK(cudaMalloc(&I.d_solid, solid_table_bytes(c->storage, I.ip.solid_blocks, c->B * c->B)));
+        I.ip.solid_tab = I.d_solid;
+        TRY(upload(c, c->d_ip + ii, &I.ip, sizeof(InstParams)));
+    }
     I.ts = ts;
     I.bs = std::move(bs);
     I.planned = std::move(planned);
@@ -1608,7 +1620,7 @@ bool footprint_kept(const Inst& I, long long n, int m) {
 sbot_status step_persistent(sbot_ctx* c, int most, int* ran) {
     *ran = 0;
     const DevPool P = pool_view(c);
-    if (!c->persist || c->staged || (P.coll & COLL_SOLID) || (c->prof_mask & 15)) return SBOT_OK;
+    if (!c->persist || c->staged || (c->prof_mask & 15)) return SBOT_OK;
     const int g = c->par[0];
     int steps = most >= c->steps_per_launch ? c->steps_per_launch : 1;  // one list of each length
     if (c->prof_mask & 16) steps = 1;
@@ -1637,6 +1649,7 @@ sbot_status step_persistent(sbot_ctx* c, int most, int* ran) {
     A.spin_ns = c->spin_ns;
     A.bulk_rounds = c->bulk_rounds;
     A.crit_items = c->crit_items;
+    A.fixed = c->groups == 1u;
     A.max_servers = c->step_grid / 4;
     for (int l = 0; l < SBOT_MAXLEV; l++) {
         const int gl = gl_of(l + 1, l);
@@ -1827,6 +1840,8 @@ void free_inst_device(Inst& I) {
     I.d_ibmcache = nullptr;
     dfree(I.d_fterm);
     I.d_fterm = nullptr;
+    dfree(I.d_solid);
+    I.d_solid = nullptr;
     I.d_latmap = nullptr;
     I.d_int = nullptr;
     I.d_qx = I.d_qy = nullptr;
@@ -2077,6 +2092,11 @@ sbot_status admit(sbot_ctx* c, int ii, const sbot_domain_desc* desc, const sbot_
         if (I.has_body) list_add(c, gl_of(I.m, I.m - 1), LK_IBM, ii, I.ip.patch_cap);
         st = refresh_groups(c);
         if (st == SBOT_OK) st = flush(c);
+    }
+    if (st == SBOT_OK && I.d_solid) {
+        launch_solid_table(c->storage, pool_view(c), int_part(I, I.m - 1), I.int_n[I.m - 1], I.d_solid,
+                           I.ip.solid_blocks, I.m - 1, c->s);
+        if (cudaGetLastError() != cudaSuccess) st = fail(c, SBOT_ERR_CUDA, "the solid's table: launch failed");
     }
     if (st == SBOT_OK) st = reset_state(c, ii);
     if (st == SBOT_OK) st = end_frame(c);

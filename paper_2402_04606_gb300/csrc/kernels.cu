@@ -121,6 +121,19 @@ __global__ void __launch_bounds__(1024) k_collide_init(const __grid_constant__ D
     for (int q = 0; q < 9; q++) Sto<S>::template st<C>(fpost, ((size_t)slot * 9 + q) * BB + cell, q, f[q], ip.dref);
 }
 
+template <class C>
+__global__ void __launch_bounds__(1024) k_solid_table(const __grid_constant__ DevPool P, const int* __restrict__ list, int n,
+                                                      void* tab, int blocks, int level) {
+    const int slot = list[blockIdx.x], B = P.B, BB = B * B, cell = threadIdx.x;
+    if ((int)blockIdx.x >= n || !(P.slot_flags[slot] & SLOTF_SOLID)) return;
+    const size_t blk = (size_t)P.slot_parent[slot];
+    if (blk >= (size_t)blocks) return;
+    C* const coef = (C*)tab;
+    unsigned* const word = (unsigned*)(coef + (size_t)blocks * BB * 16);
+    solid_fill<C>(P.inst[P.slot_inst[slot]], level, P.slot_ox[slot] + cell % B, P.slot_oy[slot] + cell / B, cell, BB,
+                  coef + blk * 16 * BB, word + blk * BB);
+}
+
 template <class S>
 __global__ void __launch_bounds__(1024) k_c2f(const __grid_constant__ DevPool P, const int* __restrict__ list, const int* __restrict__ pn,
                                               const S* __restrict__ fc, S* __restrict__ ff) {
@@ -673,6 +686,19 @@ void launch_collide_init(int storage, const DevPool& P, const int* list, int n, 
         else
             k_collide_init<S, C, 0><<<n, P.B * P.B, 0, s>>>(P, list, n, (const S*)fpre, (S*)fpost, level);
     });
+}
+
+size_t solid_table_bytes(int storage, int blocks, int BB) {
+    return storage == 0 ? SolidTab<double>::bytes(blocks, BB) : SolidTab<float>::bytes(blocks, BB);
+}
+
+void launch_solid_table(int storage, const DevPool& P, const int* list, int n, void* tab, int blocks, int level,
+                        sbot_stream_t s) {
+    if (n <= 0) return;
+    if (storage == 0)
+        k_solid_table<double><<<n, P.B * P.B, 0, s>>>(P, list, n, tab, blocks, level);
+    else
+        k_solid_table<float><<<n, P.B * P.B, 0, s>>>(P, list, n, tab, blocks, level);
 }
 
 void launch_c2f(int storage, const DevPool& P, const int* list, const int* pn, int cap, const void* fcoarse,

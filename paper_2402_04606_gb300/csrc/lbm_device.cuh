@@ -477,21 +477,36 @@ __device__ __forceinline__ bool mask_bit(const DevPool& P, int slot, int cell) {
 
 __device__ __forceinline__ int wrapi(int v, int n) { return ((v % n) + n) % n; }
 
+// what a moving wall side adds to direction q, 2 w_q rho0 (c_q . u_w) / c_s^2
+// (rounded by itself: the same value read from SlotMeta or formed where it is added)
+__device__ __forceinline__ double wall_gain(const InstParams& ip, int side, int q) {
+    return __dmul_rn(6.0 * Wq<double>(q) * ip.rho0, CXq(q) * ip.uwall[side][0] + CYq(q) * ip.uwall[side][1]);
+}
+
 // Where a sweep finds the per-block data of the slot it updates: the pool's
 // tables (MetaG), or a copy in shared memory (MetaS over a SlotMeta), which a
 // task of the persistent step kernel reads before it waits for the phases it
 // depends on (none of this data changes during a step).  Both give the same
 // values, so the arithmetic is the same either way.
+template <class C>
 struct SlotMeta {
-    int slot, type, flags, inst, ox, oy;
+    int slot, type, flags, inst, ox, oy, parent;
     int nb[9], nbt[9];        // neighbour slots (-1: none) and their types
     int child[4], childt[4];  // quarter children on the next level (-1: none) and their types
+    // what else a sweep would read from the instance after its wait, when the
+    // SM's cached lines are gone: 1 / tau of the level; the kind of each domain
+    // side the block touches (-1: none) and a wall side's addend per direction
+    C om;
+    int kind[4];
+    C wall[4][9];
 };
 struct MetaG {
+    static constexpr bool shared = false;
     const DevPool& P;
     int s;
     __device__ __forceinline__ int slot() const { return s; }
     __device__ __forceinline__ int flags() const { return P.slot_flags[s]; }
+    __device__ __forceinline__ int parent() const { return P.slot_parent[s]; }
     __device__ __forceinline__ int ox() const { return P.slot_ox[s]; }
     __device__ __forceinline__ int oy() const { return P.slot_oy[s]; }
     __device__ __forceinline__ int nb(int k) const { return P.nbr[s * 9 + k]; }
@@ -499,10 +514,13 @@ struct MetaG {
     __device__ __forceinline__ int child(int k) const { return P.slot_child[s * 4 + k]; }
     __device__ __forceinline__ int childt(int, int c) const { return P.slot_type[c]; }
 };
+template <class C>
 struct MetaS {
-    const SlotMeta* m;
+    static constexpr bool shared = true;
+    const SlotMeta<C>* m;
     __device__ __forceinline__ int slot() const { return m->slot; }
     __device__ __forceinline__ int flags() const { return m->flags; }
+    __device__ __forceinline__ int parent() const { return m->parent; }
     __device__ __forceinline__ int ox() const { return m->ox; }
     __device__ __forceinline__ int oy() const { return m->oy; }
     __device__ __forceinline__ int nb(int k) const { return m->nb[k]; }
@@ -511,9 +529,24 @@ struct MetaS {
     __device__ __forceinline__ int childt(int k, int) const { return m->childt[k]; }
 };
 
-// one warp: the data of `slot` into m (two dependent rounds of loads)
-__device__ __forceinline__ void load_meta(const DevPool& P, int slot, SlotMeta& m) {
+// one warp: the data of `slot` (of `level`) into m (two dependent rounds of loads)
+template <class C>
+__device__ __forceinline__ void load_meta(const DevPool& P, int slot, int level, SlotMeta<C>& m) {
     const int lane = threadIdx.x & 31;
+    const InstParams& ip = P.inst[P.slot_inst[slot]];
+    if (lane == 19) m.om = (C)1 / (C)ip.tau[level];
+    if (P.slot_flags[slot] & SLOTF_EDGE) {
+        const int ox = P.slot_ox[slot], oy = P.slot_oy[slot], nxl = ip.nx0 << level, nyl = ip.ny0 << level;
+        if (lane < 4) {
+            const bool at = lane == SIDE_W ? ox == 0 : lane == SIDE_E ? ox + P.B == nxl : lane == SIDE_S ? oy == 0
+                                                                                                 : oy + P.B == nyl;
+            m.kind[lane] = at && ip.bc[lane] != BCK_PERIODIC ? ip.bc[lane] : -1;
+        }
+        for (int e = lane; e < 36; e += 32) {
+            const int k = e / 9, q = e % 9;
+            m.wall[k][q] = (C)wall_gain(ip, k, q);
+        }
+    }
     if (lane < 9) {
         const int ns = P.nbr[slot * 9 + lane];
         m.nb[lane] = ns;
@@ -533,6 +566,8 @@ __device__ __forceinline__ void load_meta(const DevPool& P, int slot, SlotMeta& 
         m.ox = P.slot_ox[slot];
     } else if (lane == 17) {
         m.oy = P.slot_oy[slot];
+    } else if (lane == 18) {
+        m.parent = P.slot_parent[slot];
     }
 }
 
@@ -542,61 +577,47 @@ __device__ __forceinline__ int lat_slot(const DevPool& P, const InstParams& ip, 
     return ip.latmap[ip.latmap_off[level] + (long long)(gy / P.B) * ip.nbx[level] + gx / P.B];
 }
 
-// Half-way bounce-back from a wall side (reading R15): the population that
-// left cell (ox, oy) toward the wall returns reversed, plus the momentum of
-// the moving wall, 2 w_q rho0 (c_q . u_w) / c_s^2 (the same on deviations:
-// opposite directions share w_q).
-template <class S, class C>
-__device__ C wall_bounce(const DevPool& P, const S* fin, const InstParams& ip, int level, int ox, int oy, int q,
-                         int side) {
-    const int s = lat_slot(P, ip, level, ox, oy);
-    if (s < 0) {
-        atomicOr(P.err, ERRB_NOSOURCE);
-        return (C)0;
-    }
-    const int o = flipX(flipY(q)), B = P.B;
-    const C a = Sto<S>::template ld<C>(fin, ((size_t)s * 9 + o) * B * B + (oy - P.slot_oy[s]) * B + (ox - P.slot_ox[s]), o,
-                                       ip.dref);
-    const double mw = 6.0 * Wq<double>(q) * ip.rho0 * (CXq(q) * ip.uwall[side][0] + CYq(q) * ip.uwall[side][1]);
-    return a + (C)mw;
-}
-
-// Pull from outside the domain (non-periodic side), reading R2: the y-side
-// rule first, then the x-side rule; periodic axes wrap.  (gx, gy) is the
-// source of direction q; the cell pulling is (gx, gy) + c_q.
-template <class S, class C>
-__device__ __noinline__ C pull_boundary(const DevPool& P, const S* fin, const InstParams& ip, int level, int gx,
-                                        int gy, int q) {
-    const int ox = gx + CXq(q), oy = gy + CYq(q);
-    int nxl = ip.nx0 << level, nyl = ip.ny0 << level;
-    if (ip.periodic_y) gy = wrapi(gy, nyl);
-    if (ip.periodic_x) gx = wrapi(gx, nxl);
-    if (gy < 0 || gy >= nyl) {
-        int side = gy < 0 ? SIDE_S : SIDE_N;
-        int edge = gy < 0 ? 0 : nyl - 1;
-        int k = ip.bc[side];
+// Pull of direction q into cell (x, y) of the slot mt describes from outside
+// the domain (non-periodic side), reading R2: the y-side rule first, then the
+// x-side rule.  A wall side (half-way bounce-back, reading R15) returns the
+// population that left the cell toward it reversed, plus the momentum of the
+// moving wall, 2 w_q rho0 (c_q . u_w) / c_s^2 (the same on deviations: opposite
+// directions share w_q).  Every source lies in the block or a neighbour of it, so
+// it is found through the neighbour table, which a sweep's task holds in shared
+// memory (through the lattice map, a chain of three loads from L2: a 304^2 cavity
+// with walls and a bounce-back cylinder took @W@).
+template <class S, class C, class M>
+__device__ __noinline__ C pull_boundary(const DevPool& P, M mt, const S* fin, const InstParams& ip, int level, int x,
+                                        int y, int q) {
+    const int B = P.B, BB = B * B, ox = mt.ox(), oy = mt.oy();
+    const int nxl = ip.nx0 << level, nyl = ip.ny0 << level;
+    int lx = x - CXq(q), ly = y - CYq(q);
+    auto wall = [&](int side) -> C {
+        const int o = flipX(flipY(q));
+        const C a = Sto<S>::template ld<C>(fin, ((size_t)mt.slot() * 9 + o) * BB + y * B + x, o, ip.dref);
+        return a + (C)wall_gain(ip, side, q);
+    };
+    if (!ip.periodic_y && (oy + ly < 0 || oy + ly >= nyl)) {
+        const int side = oy + ly < 0 ? SIDE_S : SIDE_N, k = ip.bc[side];
         if (k == BCK_INLET) return feq_s<S, C>(q, (C)ip.rho0, (C)ip.uin_x, (C)ip.uin_y);
-        if (k == BCK_WALL) return wall_bounce<S, C>(P, fin, ip, level, ox, oy, q, side);
-        gy = edge;
+        if (k == BCK_WALL) return wall(side);
+        ly = (side == SIDE_S ? 0 : nyl - 1) - oy;
         if (k == BCK_SYMMETRY) q = flipY(q);
     }
-    if (gx < 0 || gx >= nxl) {
-        int side = gx < 0 ? SIDE_W : SIDE_E;
-        int edge = gx < 0 ? 0 : nxl - 1;
-        int k = ip.bc[side];
+    if (!ip.periodic_x && (ox + lx < 0 || ox + lx >= nxl)) {
+        const int side = ox + lx < 0 ? SIDE_W : SIDE_E, k = ip.bc[side];
         if (k == BCK_INLET) return feq_s<S, C>(q, (C)ip.rho0, (C)ip.uin_x, (C)ip.uin_y);
-        if (k == BCK_WALL) return wall_bounce<S, C>(P, fin, ip, level, ox, oy, q, side);
-        gx = edge;
+        if (k == BCK_WALL) return wall(side);
+        lx = (side == SIDE_W ? 0 : nxl - 1) - ox;
         if (k == BCK_SYMMETRY) q = flipX(q);
     }
-    int s = lat_slot(P, ip, level, gx, gy);
+    const int dx = lx < 0 ? -1 : (lx >= B ? 1 : 0), dy = ly < 0 ? -1 : (ly >= B ? 1 : 0);
+    const int s = mt.nb((dy + 1) * 3 + dx + 1);
     if (s < 0) {
         atomicOr(P.err, ERRB_NOSOURCE);
         return (C)0;
     }
-    int B = P.B;
-    return Sto<S>::template ld<C>(fin, ((size_t)s * 9 + q) * B * B + (gy - P.slot_oy[s]) * B + (gx - P.slot_ox[s]), q,
-                                  ip.dref);
+    return Sto<S>::template ld<C>(fin, ((size_t)s * 9 + q) * BB + (ly - dy * B) * B + (lx - dx * B), q, ip.dref);
 }
 
 // The volumetric merge (Sec. 2.4 step 6, reading R3c): population q of
@@ -640,7 +661,49 @@ __device__ __forceinline__ C pull_int(const DevPool& P, M mt, const S* fin, cons
         return Sto<S>::template ld<C>(fin, ((size_t)ns * 9 + q) * B * B + (sy - dy * B) * B + (sx - dx * B), q,
                                       ip.dref);
     }
-    return pull_boundary<S, C>(P, fin, ip, level, mt.ox() + sx, mt.oy() + sy, q);
+    if constexpr (M::shared) {
+        // pull_boundary's rules, inlined: no call between the cell's loads, so
+        // that they are in flight together.  (What comes in through an inlet side
+        // is not used: its cells are reset after streaming.)
+        const auto& m = *mt.m;
+        int r = q, wall = -1;
+        bool inlet = false;
+        if (sy < 0 || sy >= B) {
+            const int side = sy < 0 ? SIDE_S : SIDE_N, kd = m.kind[side];
+            if (kd >= 0) {
+                inlet = kd == BCK_INLET;
+                wall = kd == BCK_WALL ? side : -1;
+                sy = sy < 0 ? 0 : B - 1;
+                if (kd == BCK_SYMMETRY) r = flipY(r);
+            }
+        }
+        if (wall < 0 && (sx < 0 || sx >= B)) {
+            const int side = sx < 0 ? SIDE_W : SIDE_E, kd = m.kind[side];
+            if (kd >= 0) {
+                inlet |= kd == BCK_INLET;
+                wall = kd == BCK_WALL ? side : -1;
+                sx = sx < 0 ? 0 : B - 1;
+                if (kd == BCK_SYMMETRY) r = flipX(r);
+            }
+        }
+        if (inlet) return (C)0;
+        C add = 0;
+        if (wall >= 0) {
+            add = m.wall[wall][r];
+            r = flipX(flipY(r));
+            sx = x, sy = y;
+        }
+        dx = sx < 0 ? -1 : (sx >= B ? 1 : 0);
+        dy = sy < 0 ? -1 : (sy >= B ? 1 : 0);
+        ns = mt.nb((dy + 1) * 3 + dx + 1);
+        if (ns < 0) {
+            atomicOr(P.err, ERRB_NOSOURCE);
+            return (C)0;
+        }
+        return Sto<S>::template ld<C>(fin, ((size_t)ns * 9 + r) * B * B + (sy - dy * B) * B + (sx - dx * B), r, ip.dref) +
+               add;
+    }
+    return pull_boundary<S, C, M>(P, mt, fin, ip, level, x, y, q);
 }
 template <class S, class C>
 __device__ __forceinline__ C pull_int(const DevPool& P, const S* fin, const S* ffine, bool mailbox, int slot,
@@ -707,6 +770,51 @@ __device__ __noinline__ bool solid_links(const DevPool& P, const S* fin, int slo
     return true;
 }
 
+// The links of solid_links worked out once per topology (solids do not move, nor
+// does the refinement around them): per cell of a block near a solid one word --
+// bit q: the source of direction q is solid; bit 9 + q: its t < 1/2 form applies;
+// bit 20: the cell is solid -- and per direction the form's two factors in the
+// compute type.  A block's entry is the index its slot_parent holds.
+#define SOLID_CELL (1u << 20)
+template <class C>
+struct SolidTab {
+    static __host__ __device__ size_t bytes(int blocks, int BB) {
+        return (size_t)blocks * BB * (sizeof(C) * 16 + sizeof(unsigned));
+    }
+    const C* coef;  // [block][q - 1][2][cell]
+    const unsigned* word;  // [block][cell]
+    __device__ SolidTab(const void* p, int blocks, int BB)
+        : coef((const C*)p), word((const unsigned*)((const C*)p + (size_t)blocks * BB * 16)) {}
+};
+template <class C>
+__device__ void solid_fill(const InstParams& ip, int level, int gx, int gy, int cell, int BB, C* coef,
+                           unsigned* word) {
+    const double px = gx + 0.5, py = gy + 0.5;
+    const int nxl = ip.nx0 << level, nyl = ip.ny0 << level;
+    unsigned w = in_solid(ip, px, py) ? SOLID_CELL : 0u;
+    for (int q = 1; q < 9; q++) {
+        const int cx = CXq(q), cy = CYq(q);
+        C c0 = 0, c1 = 0;
+        if (!(w & SOLID_CELL) && in_solid(ip, px - cx, py - cy)) {
+            const double t = link_outside(ip, px, py, (double)-cx, (double)-cy);
+            const int fx = gx + cx, fy = gy + cy;
+            const bool far_fluid = (ip.periodic_x || (fx >= 0 && fx < nxl)) &&
+                                   (ip.periodic_y || (fy >= 0 && fy < nyl)) && !in_solid(ip, px + cx, py + cy);
+            w |= 1u << q;
+            c0 = (C)(2.0 * t);
+            if (t < 0.5 && far_fluid) {
+                w |= 1u << (9 + q);
+                c1 = (C)(1.0 - 2.0 * t);
+            } else {
+                c1 = (C)(1.0 - 1.0 / (2.0 * t));
+            }
+        }
+        coef[(size_t)(2 * (q - 1)) * BB + cell] = c0;
+        coef[(size_t)(2 * (q - 1) + 1) * BB + cell] = c1;
+    }
+    word[cell] = w;
+}
+
 template <class C>
 __device__ __forceinline__ bool inlet_cell(const InstParams& ip, int level, int gx, int gy) {
     int nxl = ip.nx0 << level, nyl = ip.ny0 << level;
@@ -766,19 +874,58 @@ __device__ __forceinline__ void fused_cell(const DevPool& P, M mt, const S* fin,
     C f[9];
     const int flags = mt.flags();
     const bool mailbox = (flags & SLOTF_MAILBOX) != 0;
+    unsigned links = 0;  // (SOLID: only in contexts holding a solid; the code costs every kernel that contains it)
+    const C* coef = nullptr;
+    if constexpr (SOLID) {
+        if (flags & SLOTF_SOLID) {
+            const SolidTab<C> tab(ip.solid_tab, ip.solid_blocks, BB);
+            const size_t blk = (size_t)mt.parent();
+            links = tab.word[blk * BB + cell];
+            coef = tab.coef + blk * 16 * BB + cell;
+        }
+    }
 #pragma unroll
     for (int q = 0; q < 9; q++) f[q] = pull_int<S, C, M>(P, mt, fin, ffine, mailbox, ip, level, x, y, q);
-    if constexpr (SOLID) {  // only in contexts holding a solid: the code costs every kernel that contains it
-        if ((flags & SLOTF_SOLID) && !solid_links<S, C>(P, fin, slot, ip, level, x, y, f)) return;
+    if constexpr (SOLID) {
+        if (links & SOLID_CELL) return;  // left as it is
+        if (links != 0) {
+            C g[9];
+#pragma unroll
+            for (int q = 0; q < 9; q++) g[q] = f[q];
+            const size_t own = (size_t)slot * 9 * BB + cell;
+#pragma unroll
+            for (int q = 1; q < 9; q++) {
+                constexpr int opp[9] = {0, 3, 4, 1, 2, 7, 8, 5, 6};
+                if (!((links >> q) & 1u)) continue;
+                const C c0 = coef[(size_t)(2 * (q - 1)) * BB], c1 = coef[(size_t)(2 * (q - 1) + 1) * BB];
+                const C a = Sto<S>::template ld<C>(fin, own + (size_t)opp[q] * BB, opp[q], ip.dref);
+                if ((links >> (9 + q)) & 1u)
+                    f[q] = c0 * a + c1 * g[opp[q]];
+                else
+                    f[q] = a / c0 + c1 * Sto<S>::template ld<C>(fin, own + (size_t)q * BB, q, ip.dref);
+            }
+        }
     }
-    if ((flags & SLOTF_EDGE) && inlet_cell<C>(ip, level, mt.ox() + x, mt.oy() + y)) {
+    bool inlet = false;
+    C om;
+    if constexpr (M::shared) {
+        const auto& m = *mt.m;
+        om = m.om;
+        if (flags & SLOTF_EDGE)
+            inlet = (x == 0 && m.kind[SIDE_W] == BCK_INLET) || (x == B - 1 && m.kind[SIDE_E] == BCK_INLET) ||
+                    (y == 0 && m.kind[SIDE_S] == BCK_INLET) || (y == B - 1 && m.kind[SIDE_N] == BCK_INLET);
+    } else {
+        om = (C)1 / (C)ip.tau[level];
+        inlet = (flags & SLOTF_EDGE) && inlet_cell<C>(ip, level, mt.ox() + x, mt.oy() + y);
+    }
+    if (inlet) {
 #pragma unroll
         for (int q = 0; q < 9; q++) f[q] = feq_s<S, C>(q, (C)ip.rho0, (C)ip.uin_x, (C)ip.uin_y);
     }
     // (16-bit storage keeps the forced form at zero force: its two forms contract
     // to different fmas, and one unit of a 16-bit store in every cell's history
     // is more than a change of schedule may make; the others agree bit for bit)
-    collide_k<COLL, C, sizeof(S) == 2, DevTrait<S>::value, sizeof(S) == 4>(f, (C)1 / (C)ip.tau[level], (C)0, (C)0, ip);
+    collide_k<COLL, C, sizeof(S) == 2, DevTrait<S>::value, sizeof(S) == 4>(f, om, (C)0, (C)0, ip);
 #pragma unroll
     for (int q = 0; q < 9; q++) Sto<S>::template st<C>(fout, ((size_t)slot * 9 + q) * BB + cell, q, f[q], ip.dref);
     if (fhalo != nullptr && mailbox) {

@@ -73,6 +73,8 @@ struct InstParams {
     double uwall[4][2];                         // velocity of each wall side
     int solid;                                  // 0 none, 1 circle, 2 half-plane y < y0 (finest level)
     double sol[3];
+    const void* solid_tab;                      // the solid's links (SolidTab), nullptr without a solid
+    int solid_blocks;                           // its blocks
     double ramp_as, ramp_rate, ramp_t1, t_ref;  // motion 3 (pitch-up ramp)
     double asym_xi, accel_frac;                 // motion 4 (triangular pitch)
     void* patch;     // force patch, compute type, [2][patch_cap]
@@ -106,7 +108,8 @@ struct DevPool {
     const int* slot_ox;  // cell origin of the block at its level
     const int* slot_oy;
     const int* slot_flags;
-    const int* slot_parent;  // ST_GF: parent slot (ST_INT, level - 1), else -1
+    const int* slot_parent;  // ST_GF: parent slot (ST_INT, level - 1); a block near a solid: its entry in the
+                             // links' table; else -1
     const int* slot_child;   // [S][4]: ST_INT: the slots of its 4 quarter blocks on level + 1 ((qy * 2 + qx)), else -1
     const unsigned* slot_mask;  // [S][mask_words]: halo / mailbox cells
     const InstParams* inst;
@@ -151,6 +154,10 @@ void launch_fused(int storage, const DevPool& P, const int* list, const int* pn,
                   sbot_stream_t s, void* fhalo = nullptr);
 void launch_collide_init(int storage, const DevPool& P, const int* list, int n, const void* fpre, void* fpost,
                          int level, sbot_stream_t s);
+// the links' table of an instance with a solid: the blocks near it among the n finest ones of `list`
+void launch_solid_table(int storage, const DevPool& P, const int* list, int n, void* tab, int blocks, int level,
+                        sbot_stream_t s);
+size_t solid_table_bytes(int storage, int blocks, int BB);
 void launch_c2f(int storage, const DevPool& P, const int* list, const int* pn, int cap, const void* fcoarse,
                 void* ffine, sbot_stream_t s);
 // the poses of one coarse step of every moving body in an instance list (Sec. 3.6)
@@ -243,6 +250,7 @@ struct StepArgs {
     long long spin_ns;        // longest wait for a dependency before the launch gives up (ERRB_TIMEOUT)
     int bulk_rounds;          // vector rounds per bulk task
     int crit_items;           // > 0: at most this many list items per task of a critical fused phase
+    int fixed;                // 1: every task has a fixed owner (all instances have one level)
     int max_servers;          // most thread blocks set apart for one body's IBM each (more bodies: no block is)
     int body_count[SBOT_MAXLEV];  // per group, the index of its body list's length, -1 none
     // phase trace (nullptr: off): device ns of each phase's first task start

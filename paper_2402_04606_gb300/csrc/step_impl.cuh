@@ -42,6 +42,9 @@
 #pragma once
 #include "lbm_device.cuh"
 
+#ifndef STEP_SOLID
+#define STEP_SOLID true
+#endif
 namespace {
 
 enum { STEP_EXIT = 0, STEP_RUN = 1 };
@@ -98,12 +101,18 @@ struct TaskShape {
         return parts > 1 ? n * parts : (n + per * rounds - 1) / (per * rounds);
     }
 };
+// A launch of fixed owners (StepArgs::fixed) cuts a sweep into at most one task
+// per thread block: handing out costs nothing there, so a short list is spread
+// over all of them.
 template <class S, int B>
-__device__ __forceinline__ TaskShape task_shape(const StepArgs& A, const StepPhase& ph, int n, bool vec, int T) {
+__device__ __forceinline__ TaskShape task_shape(const StepArgs& A, const StepPhase& ph, int n, bool vec, int T,
+                                                int grid) {
     TaskShape t{fused_items<S, B>(vec, T), 1, 1};
-    const int grid = gridDim.x;
     const long long fill = (long long)t.per * grid;  // items of one filling of every thread block
-    if (ph.bulk || n > 8 * fill) {
+    if (A.fixed) {
+        t.rounds = (int)((n + fill - 1) / fill);
+        if (n < fill) t.per = (n + grid - 1) / grid;
+    } else if (ph.bulk || n > 8 * fill) {
         const long long waves = (n + fill * A.bulk_rounds - 1) / (fill * A.bulk_rounds);
         t.rounds = (int)((n + fill * waves - 1) / (fill * waves));
     } else if (A.crit_items > 0) {
@@ -121,12 +130,12 @@ __device__ __forceinline__ TaskShape task_shape(const StepArgs& A, const StepPha
 
 // tasks of phase p at this launch (from the device list lengths)
 template <class S, int B>
-__device__ int step_ntasks(const DevPool& P, const StepArgs& A, const StepPhase& ph, int T) {
+__device__ int step_ntasks(const DevPool& P, const StepArgs& A, const StepPhase& ph, int T, int grid) {
     const int n = A.counts[ph.count_idx];
     if (n <= 0) return 0;
     switch (ph.kind) {
     case PH_FUSED: {
-        return task_shape<S, B>(A, ph, n, fused_vec<S, B>(A, ph, n, P.coll), T).tasks(n);
+        return task_shape<S, B>(A, ph, n, fused_vec<S, B>(A, ph, n, P.coll), T, grid).tasks(n);
     }
     case PH_C2F: {
         const int per = T >= B * B ? T / (B * B) : 1;
@@ -153,9 +162,12 @@ __device__ __forceinline__ void for_cells(int n, int i0, int k, int BB, F&& fn) 
 // their types, children) into shared memory, which it may do before the
 // phases it depends on have finished: after the gate only the population
 // and force loads remain on its path.
+// key: which task's blocks' data the shared memory holds (a thread block of a
+// launch of fixed owners runs the same task in every step, and reads them once).
 template <class S, class C, int B, int COLL, class G>
-__device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, G& gate) {
-    __shared__ SlotMeta meta[STEP_META_MAX];
+__device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, int grid, int2& key,
+                           G& gate) {
+    __shared__ SlotMeta<C> meta[STEP_META_MAX];
     const int n = A.counts[ph.count_idx];
     const int* list = A.lists + ph.list_off;
     const S* fin = step_buf<S>(A, ph.fin);
@@ -164,19 +176,21 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
     S* fhalo = ph.fold ? step_buf<S>(A, ph.ffine) : nullptr;  // the coarse-to-fine copy rides on this sweep
     const int T = blockDim.x;
     const bool vec = fused_vec<S, B>(A, ph, n, P.coll);
-    const TaskShape sh = task_shape<S, B>(A, ph, n, vec, T);
+    const TaskShape sh = task_shape<S, B>(A, ph, n, vec, T, grid);
     const int per = sh.per, rounds = sh.rounds;
     if (rounds == 1 && !vec && per <= STEP_META_MAX && per <= T / 32) {
         const int i0 = sh.parts > 1 ? local / sh.parts : local * per, ne = min(n, i0 + per), w = threadIdx.x >> 5;
         // its cells: those of its items, or a part of one item's
         const int len = sh.parts > 1 ? B * B / sh.parts : (ne - i0) * B * B;
         const int c0 = sh.parts > 1 ? (local - i0 * sh.parts) * len : 0;
-        if (i0 + w < ne) load_meta(P, list[i0 + w], meta[w]);
+        const bool held = key.x == ph.list_off && key.y == local;
+        if (!held && i0 + w < ne) load_meta<C>(P, list[i0 + w], ph.level, meta[w]);
         if (!gate(true)) return;
+        if (threadIdx.x == 0) key = make_int2(ph.list_off, local);
         for (int c = c0 + threadIdx.x; c < c0 + len; c += T) {
-            const SlotMeta& m = meta[c / (B * B)];
+            const SlotMeta<C>& m = meta[c / (B * B)];
             const int cell = c % (B * B);
-            fused_cell<S, C, COLL, false, MetaS>(P, MetaS{&m}, fin, fout, ffine, m.type, P.inst[m.inst], ph.level,
+            fused_cell<S, C, COLL, STEP_SOLID, MetaS<C>>(P, MetaS<C>{&m}, fin, fout, ffine, m.type, P.inst[m.inst], ph.level,
                                                  cell % B, cell / B, fhalo);
         }
         return;
@@ -198,7 +212,7 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
         }
         for_cells(ne, i0, per, B * B, [&](int item, int cell) {
             const int slot = list[item];
-            fused_cell<S, C, COLL, false>(P, fin, fout, ffine, slot, P.slot_type[slot], P.inst[P.slot_inst[slot]],
+            fused_cell<S, C, COLL, STEP_SOLID>(P, fin, fout, ffine, slot, P.slot_type[slot], P.inst[P.slot_inst[slot]],
                                           ph.level, cell % B, cell / B, fhalo);
         });
     }
@@ -213,15 +227,15 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
 // An IBM task waits before its stores for the sweep of its sub-step
 // (ph.after): await() by one warp, swept() by all after a barrier (ibm_run).
 template <class S, class C, int B, int COLL, class G, class G1, class G2>
-__device__ void step_task(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, unsigned char* smraw,
-                          IbmShared& sh, G& gate, G1& await, G2& swept) {
+__device__ void step_task(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, int grid, int2& key,
+                          unsigned char* smraw, IbmShared& sh, G& gate, G1& await, G2& swept) {
     const int* list = A.lists + ph.list_off;
     if (A.counts[ph.count_idx] <= 0) {  // the empty task of a phase with no work
         gate(false);
         return;
     }
     switch (ph.kind) {
-    case PH_FUSED: step_fused<S, C, B, COLL>(P, A, ph, local, gate); break;
+    case PH_FUSED: step_fused<S, C, B, COLL>(P, A, ph, local, grid, key, gate); break;
     case PH_IBM:
         ibm_run<S, C, COLL>(P, list[local], step_buf<S>(A, ph.fin), step_buf<S>(A, ph.fout), ph.level, 0, 1, ph.arg,
                             smraw, sh, gate, await, swept);
@@ -351,7 +365,8 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
     __shared__ int wtot[32];
     // the scheduler's state lives in shared memory, so that no register is
     // held across a task (the vector sweep needs all of them)
-    __shared__ int s_cmd, s_phase, s_local, s_last, s_ncp, s_nbulk, s_bulk_left, s_turn;
+    __shared__ int s_cmd, s_phase, s_local, s_last, s_ncp, s_nbulk, s_bulk_left, s_turn, s_next;
+    __shared__ int2 s_key;  // the sweep task whose blocks' data are held (step_fused)
     __shared__ int s_wait, s_go;  // the claimed critical phase to wait for (-1: none), the wait's outcome
     __shared__ int s_body[SBOT_MAXLEV + 1];  // first server of each group's bodies, their number
     const int tid = threadIdx.x, nph = A.nph;
@@ -372,11 +387,22 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
         }
         s_body[SBOT_MAXLEV] = n <= A.max_servers ? n : 0;
         s_turn = 0;
+        s_next = -1;
+        s_key = make_int2(-1, -1);
         sh.geo_inst = -1;
     }
     __syncthreads();
     const int nsrv = s_body[SBOT_MAXLEV];
     const bool server = (int)blockIdx.x < nsrv;
+    const int workers = gridDim.x - nsrv;
+    // Fixed owners: where every instance has one level, the phases of a step
+    // form one chain, and a task taken early only waits.  Each thread block then
+    // walks the list in order and runs the tasks that are its own by number (a
+    // sweep's from the first thread block on, the next sweep's after them, the
+    // others' from the last one back): no hand-out, whose four dependent L2 round
+    // trips were most of a short step, and a sweep's thread block keeps its blocks'
+    // data.  (In order and all resident, so the earliest unfinished task always
+    // runs.)
     auto served = [&](const StepPhase& ph) { return nsrv > 0 && ph.kind == PH_IBM && A.counts[ph.count_idx] > 0; };
 
     // task counts from this launch's list lengths (a critical phase with no
@@ -385,13 +411,13 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
     // compacted in order; the bulk queue's prefix sums
     for (int p = tid; p < nph; p += blockDim.x) {
         const StepPhase& ph = A.ph[p];
-        int nt = step_ntasks<S, B>(P, A, ph, blockDim.x);
-        if (nt == 0 && !ph.bulk && ph.ndep > 0) nt = 1;
+        int nt = step_ntasks<S, B>(P, A, ph, blockDim.x, workers);
+        if (nt == 0 && (A.fixed || !ph.bulk) && ph.ndep > 0) nt = 1;
         ntask[p] = nt;
         deps.n[p] = ph.ndep;
         for (int k = 0; k < ph.ndep; k++) deps.d[p][k] = (unsigned short)ph.dep[k];
-        cpos[p] = (!ph.bulk && nt > 0 && served(ph) == server) ? 1 : 0;
-        bfirst[p] = ph.bulk ? nt : 0;
+        cpos[p] = ((A.fixed || !ph.bulk) && nt > 0 && served(ph) == server) ? 1 : 0;
+        bfirst[p] = ph.bulk && !A.fixed ? nt : 0;
     }
     __syncthreads();
     {
@@ -405,7 +431,7 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
     }
     for (int p = tid; p < nph; p += blockDim.x) {
         const StepPhase& ph = A.ph[p];
-        if (!ph.bulk && ntask[p] > 0 && served(ph) == server) crit[cpos[p]] = p;
+        if ((A.fixed || !ph.bulk) && ntask[p] > 0 && served(ph) == server) crit[cpos[p]] = p;
     }
     __syncthreads();
     if (A.tr_start && tid == 0) atomicMin(&A.tr_start[STEP_MAX_PHASES], global_ns());
@@ -422,6 +448,26 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
                 s_cmd = i < s_ncp ? STEP_RUN : STEP_EXIT;
                 s_phase = s_wait = i < s_ncp ? crit[i] : -1;
                 s_local = local;
+                s_go = 1;
+            }
+        } else if (A.fixed) {
+            if (threadIdx.x == 0) {
+                const int w = (int)blockIdx.x - nsrv;
+                int i = s_turn, t = s_next, q = -1;
+                for (; i < s_ncp; i++, t = -1) {
+                    q = crit[i];
+                    if (t < 0) {  // its first task of this phase
+                        const bool sweep = A.ph[q].kind == PH_FUSED;
+                        const int off = sweep && i > 0 && A.ph[crit[i - 1]].kind == PH_FUSED ? ntask[crit[i - 1]] : 0;
+                        t = sweep ? (w + workers - off % workers) % workers : workers - 1 - w;
+                    }
+                    if (t < ntask[q]) break;
+                }
+                s_turn = i;
+                s_next = t + workers;
+                s_cmd = i < s_ncp && !ld_relaxed(&ctl->abort) ? STEP_RUN : STEP_EXIT;
+                s_phase = s_wait = i < s_ncp ? q : -1;
+                s_local = t;
                 s_go = 1;
             }
         } else if (threadIdx.x < 32) {  // warp 0 decides
@@ -543,7 +589,7 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
             if ((threadIdx.x & 31) == 0 && !ok) s_go = 0;
         };
         auto swept = [&]() -> bool { return s_go != 0; };
-        step_task<S, C, B, COLL>(P, A, A.ph[s_phase], s_local, smraw, sh, gate, await, swept);
+        step_task<S, C, B, COLL>(P, A, A.ph[s_phase], s_local, workers, s_key, smraw, sh, gate, await, swept);
         __syncthreads();  // the task's writes, then its count (a release: the
                           // barrier orders every thread's writes before it)
         if (threadIdx.x == 0 && s_go) {

@@ -169,6 +169,10 @@ struct sbot_ctx {
     double* d_partials = nullptr;
     int partials_cap = 0;
     double* d_out3 = nullptr;
+    double* d_export = nullptr;  // kept dense export buffer (export_level)
+    size_t export_cap = 0;       // bytes
+    char* pin = nullptr;         // pinned memory for small read-outs (at most twice a full force history)
+    size_t pin_cap = 0;
     // concurrency: a stream per group, and per (group, level) a side stream
     // for the blocks that need not wait (created when the group first appears)
     cudaStream_t gstream[SBOT_MAXLEV] = {};
@@ -1677,10 +1681,8 @@ sbot_status step_persistent(sbot_ctx* c, int most, int* ran) {
     return SBOT_OK;
 }
 
-sbot_status check_device_error(sbot_ctx* c) {
-    int e = 0;
-    CK(cudaMemcpyAsync(&e, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->s));
-    CK(cudaStreamSynchronize(c->s));
+// the device error word's meaning, e its value
+sbot_status report_device_error(sbot_ctx* c, int e) {
     if (e == 0) return SBOT_OK;
     CK(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->s));
     std::string m = "device reported:";
@@ -1693,6 +1695,13 @@ sbot_status check_device_error(sbot_ctx* c) {
         return fail(c, SBOT_ERR_TIMEOUT, m + " a bounded device wait (a bulk copy or a step dependency) gave up");
     if (e & ERRB_NONFINITE) return fail(c, SBOT_ERR_NONFINITE, m + " non-finite populations");
     return fail(c, SBOT_ERR_STATE, m);
+}
+
+sbot_status check_device_error(sbot_ctx* c) {
+    int e = 0;
+    CK(cudaMemcpyAsync(&e, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->s));
+    CK(cudaStreamSynchronize(c->s));
+    return report_device_error(c, e);
 }
 
 // Before its first step an instance's pre-collision state lives in the buffer
@@ -1779,24 +1788,45 @@ sbot_status reset_state(sbot_ctx* c, int ii) {
     return SBOT_OK;
 }
 
-// dense export of a level of instance I: mode 0 populations, mode 1 fields
-sbot_status export_level(sbot_ctx* c, Inst& I, int level, int mode, std::vector<double>& out) {
+// Dense export of a level of instance I: mode 0 populations, mode 1 fields, the
+// `planes` planes to out[i] (nullptr: left out), `per` planes each.  The copies
+// go straight to the caller's arrays (through an array of its own and one
+// memcpy per plane, 4096^2 fields took 59 ms, now 20), and a device buffer of
+// up to EXPORT_KEPT bytes is kept for the next call: cudaMalloc and cudaFree
+// wait for the whole device.
+constexpr size_t EXPORT_KEPT = size_t(64) << 20;
+sbot_status export_level(sbot_ctx* c, Inst& I, int level, int mode, double* const* out, int n_out) {
     int nx = I.d.nx0 << level, ny = I.d.ny0 << level;
     long long plane = (long long)nx * ny;
     int planes = mode == 0 ? 9 : 3;
+    const size_t bytes = (size_t)planes * plane * sizeof(double), part = bytes / n_out;
     double* d = nullptr;
-    CK(dalloc(&d, (size_t)planes * plane));
-    out.resize((size_t)planes * plane);
-    cudaError_t e = cudaMemsetAsync(d, 0, (size_t)planes * plane * sizeof(double), c->s);
+    const bool keep = bytes <= EXPORT_KEPT;
+    if (keep && c->export_cap >= bytes) {
+        d = c->d_export;
+    } else {
+        if (keep) {
+            dfree(c->d_export);
+            c->d_export = nullptr;
+            c->export_cap = 0;
+        }
+        CK(dalloc(&d, (size_t)planes * plane));
+        if (keep) {
+            c->d_export = d;
+            c->export_cap = bytes;
+        }
+    }
+    cudaError_t e = cudaMemsetAsync(d, 0, bytes, c->s);
     if (e == cudaSuccess) {
         DevPool P = pool_view(c);
         launch_export(c->storage, P, int_part(I, level), I.int_n[level], pre_buf(c, level), fine_buf(c, I, level), level,
                       I.coarse_step == 0 ? 1 : 0, nx, d, plane, mode, c->s);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out.data(), d, out.size() * sizeof(double), cudaMemcpyDeviceToHost, c->s);
+    for (int i = 0; i < n_out && e == cudaSuccess; i++)
+        if (out[i]) e = cudaMemcpyAsync(out[i], (const char*)d + i * part, part, cudaMemcpyDeviceToHost, c->s);
     cudaError_t e2 = cudaStreamSynchronize(c->s);
-    dfree(d);
+    if (!keep) dfree(d);
     CK(e);
     CK(e2);
     return check_device_error(c);
@@ -2430,27 +2460,39 @@ sbot_status sbot_get_forces(sbot_ctx_t c, double* fx, double* fy, double* mz, in
         *n_inout = 0;
         return SBOT_OK;
     }
-    CK(cudaStreamSynchronize(c->s));
-    TRY(check_device_error(c));
     long long upto = I->coarse_step << (I->m - 1);  // forces of finest steps k < canonical time
     long long avail = upto - I->forces_read;
+    const int cnt = avail > SBOT_HIST_CAP ? 0 : (int)std::min<long long>(avail, *n_inout);
+    // the error word and the entries in one wait, through pinned memory (three
+    // waits and pageable copies took 20 us a call)
+    const size_t need = 16 + (size_t)3 * cnt * sizeof(double);
+    if (need > c->pin_cap) {
+        if (c->pin) cudaFreeHost(c->pin);
+        c->pin = nullptr;
+        c->pin_cap = 0;
+        const size_t ncap = std::max<size_t>(2 * need, size_t(1) << 16);
+        CK(cudaHostAlloc((void**)&c->pin, ncap, cudaHostAllocDefault));
+        c->pin_cap = ncap;
+    }
+    int* const err = (int*)c->pin;
+    double* const h = (double*)(c->pin + 16);
+    // the ring holds entry k at k mod capacity: at most two contiguous pieces
+    const long long k0 = I->forces_read % SBOT_HIST_CAP;
+    const long long first = std::min<long long>(cnt, SBOT_HIST_CAP - k0);
+    CK(cudaMemcpyAsync(err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->s));
+    if (cnt > 0)
+        CK(cudaMemcpyAsync(h, I->d_hist + 3 * k0, (size_t)3 * first * sizeof(double), cudaMemcpyDeviceToHost, c->s));
+    if (first < cnt)
+        CK(cudaMemcpyAsync(h + 3 * first, I->d_hist, (size_t)3 * (cnt - first) * sizeof(double),
+                           cudaMemcpyDeviceToHost, c->s));
+    CK(cudaStreamSynchronize(c->s));
+    TRY(report_device_error(c, *err));
     if (avail > SBOT_HIST_CAP) {
         I->forces_read = upto - SBOT_HIST_CAP;
         *n_inout = 0;
         return fail(c, SBOT_ERR_STATE, "force history overflowed; read forces more often");
     }
-    int cnt = (int)std::min<long long>(avail, *n_inout);
     if (cnt > 0) {
-        // the ring holds entry k at k mod capacity: at most two contiguous pieces
-        std::vector<double> h((size_t)3 * cnt);
-        long long k0 = I->forces_read % SBOT_HIST_CAP;
-        long long first = std::min<long long>(cnt, SBOT_HIST_CAP - k0);
-        CK(cudaMemcpyAsync(h.data(), I->d_hist + 3 * k0, (size_t)3 * first * sizeof(double), cudaMemcpyDeviceToHost,
-                           c->s));
-        if (first < cnt)
-            CK(cudaMemcpyAsync(h.data() + 3 * first, I->d_hist, (size_t)3 * (cnt - first) * sizeof(double),
-                               cudaMemcpyDeviceToHost, c->s));
-        CK(cudaStreamSynchronize(c->s));
         for (int i = 0; i < cnt; i++) {
             if (fx) fx[i] = h[3 * i];
             if (fy) fy[i] = h[3 * i + 1];
@@ -2471,11 +2513,8 @@ sbot_status sbot_get_fields(sbot_ctx_t c, int level, double* rho, double* ux, do
         *n_inout = plane;
         return fail(c, SBOT_ERR_ARG, "output arrays too small");
     }
-    std::vector<double> out;
-    TRY(export_level(c, *I, level, 1, out));
-    if (rho) std::memcpy(rho, out.data(), plane * sizeof(double));
-    if (ux) std::memcpy(ux, out.data() + plane, plane * sizeof(double));
-    if (uy) std::memcpy(uy, out.data() + 2 * plane, plane * sizeof(double));
+    double* const out[3] = {rho, ux, uy};
+    TRY(export_level(c, *I, level, 1, out, 3));
     *n_inout = plane;
     return SBOT_OK;
 }
@@ -2489,9 +2528,7 @@ sbot_status sbot_get_populations(sbot_ctx_t c, int level, double* f, int64_t* n_
         *n_inout = n;
         return fail(c, SBOT_ERR_ARG, "output array too small");
     }
-    std::vector<double> out;
-    TRY(export_level(c, *I, level, 0, out));
-    std::memcpy(f, out.data(), n * sizeof(double));
+    TRY(export_level(c, *I, level, 0, &f, 1));
     *n_inout = n;
     return SBOT_OK;
 }
@@ -2710,8 +2747,9 @@ sbot_status sbot_destroy(sbot_ctx_t c) {
     void* ps[] = {c->d_nbr,    c->d_inst,  c->d_level, c->d_type,   c->d_ox,       c->d_oy,   c->d_flags,
                   c->d_parent, c->d_child, c->d_mask,  c->d_ip,     c->d_ist,      c->d_err,  c->d_lists,
                   c->d_counts, c->d_jobs,  c->d_out3,  c->d_one,    c->d_partials, c->d_recs,
-                  c->d_ph[0],  c->d_ph[1], c->d_ph[2], c->d_ph[3], c->d_ctl, c->d_trace};
+                  c->d_ph[0],  c->d_ph[1], c->d_ph[2], c->d_ph[3], c->d_ctl, c->d_trace, c->d_export};
     for (void* p : ps) dfree(p);
+    if (c->pin) cudaFreeHost(c->pin);
     for (auto& I : c->inst) free_inst_device(I);
     for (int g = 0; g < 2; g++) drop_graph(c, g);
     for (int i = 0; i < 2; i++) {

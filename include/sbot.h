@@ -342,8 +342,8 @@ sbot_status sbot_get_step_trace(sbot_ctx_t ctx, int* n_inout, int* kind, int* le
  * per-level sweeps, the force sums), each phase waiting on the device for
  * the phases it depends on; level-0 blocks that depend on nothing inside the
  * step fill the thread blocks that would otherwise wait.  0 (or a context
- * that profiles kernels, stages blocks with SBOT_TUNE_STAGED or holds a
- * solid obstacle) replays the per-phase CUDA graphs instead.  Each cell's
+ * that profiles kernels or stages blocks with SBOT_TUNE_STAGED) replays the
+ * per-phase CUDA graphs instead.  Each cell's
  * arithmetic is the same either way; results are equal bit for bit when
  * both take the same cell mapping (SBOT_TUNE_VECTOR_MIN_CELLS 0 or -1, or
  * blocks of 8), else to rounding. */
@@ -387,7 +387,7 @@ sbot_status sbot_get_step_trace(sbot_ctx_t ctx, int* n_inout, int* kind, int* le
 #define SBOT_TUNE_STEPS_PER_LAUNCH 9
 /* SBOT_TUNE_VEC_WAVES (-1..64, default 8): thread blocks of a vector-kernel
  * launch, in waves of resident blocks (3 per SM): at most this many waves,
- * each block walking the launch's cell list with a grid stride; 0 or
+ * each block sweeping a contiguous part of the launch's cell list; 0 or
  * negative = one block per 4 (8 in 16-bit storage) cells of each thread,
  * every block short-lived.  Fewer, longer-lived blocks sweep a large list
  * faster (less block launch and tail); short ones leave their SMs sooner to

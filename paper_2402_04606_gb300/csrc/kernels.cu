@@ -51,6 +51,12 @@ __global__ void __launch_bounds__(1024) k_fused(const __grid_constant__ DevPool 
                                   cell % B, cell / B, fhalo);
 }
 
+// items of each thread block of a vector-kernel launch: a contiguous part of the list, in whole passes
+template <int SPC>
+__device__ __forceinline__ int vec_chunk(int n) {
+    return ((n + SPC - 1) / SPC + gridDim.x - 1) / gridDim.x * SPC;
+}
+
 // (the LES variants spill at the 80 registers that 3 blocks per SM leave;
 // at 2 blocks per SM they fit in 112 registers but measured slower on the
 // 8192^2 sweep, 3.12 against 3.89 TB/s, so they keep 3)
@@ -60,18 +66,14 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : 3)
                S* __restrict__ fout, const S* __restrict__ ffine, int level) {
     pdl_enter();
     constexpr int SPC = 256 / (B * B / 4);
-    const int n = *pn;
-    int pass = 0;
-    for (int i0 = blockIdx.x * SPC; i0 < n; i0 += gridDim.x * SPC)  // grid stride (vec_grid)
-        fused_v4_task<S, C, B, COLL, true>(P, list, n, i0, pass++, fin, fout, ffine, level);
+    const int n = *pn, len = vec_chunk<SPC>(n), i0 = blockIdx.x * len;
+    fused_vec_run<S, C, B, COLL, true, false>(P, list, min(n, i0 + len), i0, SPC, fin, fout, ffine, level);
 }
 
 // Thread blocks of a vector-kernel launch: at most `waves` waves of resident
-// blocks (3 per SM, SBOT_TUNE_VEC_WAVES, default 8), each walking the list
-// with a grid stride; waves <= 0: one block per list group.  Fewer,
-// longer-lived blocks than one per list group measured faster on the 8192^2
-// sweep (FP32 0.82 -> 0.85, BF16 0.71 -> 0.75 of the measured copy
-// bandwidth): less block launch and tail per sweep.
+// blocks (3 per SM, SBOT_TUNE_VEC_WAVES, default 8), each sweeping a contiguous
+// part of the list; waves <= 0: one block per list group.  At 4096^2, 1 / 2 / 4 /
+// 8 waves take 205 / 202 / 192 / 195 us in FP32 and 120 / 121 / 123 / 119 in BF16.
 unsigned vec_grid(unsigned want, int waves) {
     static int sms = 0;
     if (waves <= 0) return want;
@@ -94,10 +96,8 @@ __global__ void __launch_bounds__(256, 3)
                S* __restrict__ fout, const S* __restrict__ ffine, int level) {
     pdl_enter();
     constexpr int SPC = 256 / (B * B / 8);
-    const int n = *pn;
-    int pass = 0;
-    for (int i0 = blockIdx.x * SPC; i0 < n; i0 += gridDim.x * SPC)  // grid stride (vec_grid)
-        fused_v8_task<S, C, B, COLL, true, SH>(P, list, n, i0, pass++, fin, fout, ffine, level);
+    const int n = *pn, len = vec_chunk<SPC>(n), i0 = blockIdx.x * len;
+    fused_vec_run<S, C, B, COLL, true, SH>(P, list, min(n, i0 + len), i0, SPC, fin, fout, ffine, level);
 }
 
 // collision only, on pre-collision populations (the state at t = 0)

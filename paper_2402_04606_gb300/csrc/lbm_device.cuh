@@ -1018,36 +1018,16 @@ __device__ __forceinline__ uint4 ld_u4(const uint4* p) {
 // every population plane is read with one 16-byte-class load per thread; the
 // +-x shift of Eq. 10 comes from the neighbouring lane by a shuffle, and only
 // the first/last lane of a row loads its edge cell from the west/east block.
-// Neighbour slots are cached in shared memory.  Halo blocks and blocks on a
-// non-periodic side (per warp: a warp never spans two blocks) take the scalar
-// path above.
-// The kernel's work for the list items item0, item0 + 1, ... (one per
-// B * B / 4 threads of the thread block; items from n on are skipped).  pass:
-// counts a block's consecutive calls (its parity picks the neighbour table).
-// NC: the input buffer does not change during the launch (loads may take the
-// read-only path).  Contains a block-wide barrier.
+// Thread t of the B * B / 4 that sweep one plain block (fused_vec_run: interior,
+// off the domain sides, no mailbox or solid); nb: its neighbour slots.  NC: the
+// input buffer does not change during the launch (loads may take the read-only
+// path).
 template <class S, class C, int B, int COLL, bool NC>
-__device__ __forceinline__ void fused_v4_task(const DevPool& P, const int* list, int n, int item0, int pass, const S* fin, S* fout,
-                                              const S* ffine, int level, S* fhalo = nullptr) {
+__device__ __forceinline__ void fused_v4_cells(const DevPool& P, const int* nb, int slot, C om, const InstParams& ip,
+                                               const S* fin, S* fout, int t) {
     static_assert(sizeof(S) >= 4, "16-bit storage takes the 8-cell kernel");
-    constexpr int BB = B * B, TPS = BB / 4, TPR = B / 4;
-    // two copies: a warp still reading this pass's while another starts the next pass
-    __shared__ int nb2[2][STEP_MAX_THREADS / TPS][9];
-    int(*const nb)[9] = nb2[pass & 1];
-    const int ls = threadIdx.x / TPS, t = threadIdx.x % TPS;
-    const int item = item0 + ls;
-    if (t < 9) nb[ls][t] = item < n ? P.nbr[list[item] * 9 + t] : -1;
-    __syncthreads();
-    if (item >= n) return;
-    const int slot = nb[ls][4];
-    const int type = P.slot_type[slot];
-    const InstParams& ip = P.inst[P.slot_inst[slot]];
+    constexpr int BB = B * B, TPR = B / 4;
     const int y = t / TPR, x0 = (t % TPR) * 4;
-    if (type != ST_INT || (P.slot_flags[slot] & (SLOTF_EDGE | SLOTF_MAILBOX | SLOTF_SOLID))) {
-        for (int i = 0; i < 4; i++)
-            fused_cell<S, C, COLL, false>(P, fin, fout, ffine, slot, type, ip, level, x0 + i, y, fhalo);
-        return;
-    }
     C f[9][4];
     if constexpr (sizeof(S) == 4) {
         // FP32: the nine rows and the edge columns are all requested before
@@ -1063,12 +1043,12 @@ __device__ __forceinline__ void fused_v4_task(const DevPool& P, const int* list,
             const int vy = sy < 0 ? 0 : (sy >= B ? 2 : 1);
             const int ry = sy + (vy == 0 ? B : (vy == 2 ? -B : 0));
             const size_t rowoff = (size_t)q * BB + ry * B;
-            raw[q] = Vec4<S, C>::template raw<NC>(fin + (size_t)nb[ls][vy * 3 + 1] * 9 * BB + rowoff + x0);
+            raw[q] = Vec4<S, C>::template raw<NC>(fin + (size_t)nb[vy * 3 + 1] * 9 * BB + rowoff + x0);
             edge[q] = (C)0;
             if (cx == 1 && x0 == 0)
-                edge[q] = Sto<S>::template ldr<C>(fin, (size_t)nb[ls][vy * 3 + 0] * 9 * BB + rowoff + (B - 1));
+                edge[q] = Sto<S>::template ldr<C>(fin, (size_t)nb[vy * 3 + 0] * 9 * BB + rowoff + (B - 1));
             if (cx == -1 && x0 + 4 == B)
-                edge[q] = Sto<S>::template ldr<C>(fin, (size_t)nb[ls][vy * 3 + 2] * 9 * BB + rowoff);
+                edge[q] = Sto<S>::template ldr<C>(fin, (size_t)nb[vy * 3 + 2] * 9 * BB + rowoff);
         }
 #pragma unroll
         for (int q = 0; q < 9; q++) {
@@ -1098,7 +1078,7 @@ __device__ __forceinline__ void fused_v4_task(const DevPool& P, const int* list,
         const int vy = sy < 0 ? 0 : (sy >= B ? 2 : 1);
         const int ry = sy + (vy == 0 ? B : (vy == 2 ? -B : 0));
         const size_t rowoff = (size_t)q * BB + ry * B;
-        const int rs = nb[ls][vy * 3 + 1];
+        const int rs = nb[vy * 3 + 1];
         C v[4];
         Vec4<S, C>::template ld<NC>(fin + (size_t)rs * 9 * BB + rowoff + x0, q, v);
         if (cx == 0) {
@@ -1106,16 +1086,15 @@ __device__ __forceinline__ void fused_v4_task(const DevPool& P, const int* list,
             for (int i = 0; i < 4; i++) f[q][i] = v[i];
         } else if (cx == 1) {
             C left = __shfl_up_sync(0xffffffffu, v[3], 1, TPR);
-            if (x0 == 0) left = Sto<S>::template ldr<C>(fin, (size_t)nb[ls][vy * 3 + 0] * 9 * BB + rowoff + (B - 1));
+            if (x0 == 0) left = Sto<S>::template ldr<C>(fin, (size_t)nb[vy * 3 + 0] * 9 * BB + rowoff + (B - 1));
             f[q][0] = left, f[q][1] = v[0], f[q][2] = v[1], f[q][3] = v[2];
         } else {
             C right = __shfl_down_sync(0xffffffffu, v[0], 1, TPR);
-            if (x0 + 4 == B) right = Sto<S>::template ldr<C>(fin, (size_t)nb[ls][vy * 3 + 2] * 9 * BB + rowoff);
+            if (x0 + 4 == B) right = Sto<S>::template ldr<C>(fin, (size_t)nb[vy * 3 + 2] * 9 * BB + rowoff);
             f[q][0] = v[1], f[q][1] = v[2], f[q][2] = v[3], f[q][3] = right;
         }
     }
     }
-    const C om = (C)1 / (C)ip.tau[level];
 #pragma unroll
     for (int i = 0; i < 4; i++) {
         C g[9];
@@ -1167,31 +1146,13 @@ __device__ __forceinline__ float el8(const uint4& r, int k) {
 // the neighbouring lane's end value by a shuffle, the first/last lane of a row
 // its edge value from the west/east block.  The arithmetic and rounding per
 // cell are those of the 4-cell kernel, so the results equal it bit for bit.
-// The kernel's work for the list items item0, item0 + 1, ... (one per
-// B * B / 8 threads; n and NC as for fused_v4_task).  Contains a block-wide
-// barrier.
+// Thread t of B * B / 8; nb and NC as for fused_v4_cells.
 template <class S, class C, int B, int COLL, bool NC, bool SH>
-__device__ __forceinline__ void fused_v8_task(const DevPool& P, const int* list, int n, int item0, int pass, const S* fin, S* fout,
-                                              const S* ffine, int level, S* fhalo = nullptr) {
+__device__ __forceinline__ void fused_v8_cells(const DevPool& P, const int* nb, int slot, C om, const InstParams& ip,
+                                               const S* fin, S* fout, int t) {
     static_assert(sizeof(S) == 2, "the 8-cell kernel is for 16-bit storage");
-    constexpr int BB = B * B, TPS = BB / 8, TPR = B / 8;
-    // two copies: a warp still reading this pass's while another starts the next pass
-    __shared__ int nb2[2][STEP_MAX_THREADS / TPS][9];
-    int(*const nb)[9] = nb2[pass & 1];
-    const int ls = threadIdx.x / TPS, t = threadIdx.x % TPS;
-    const int item = item0 + ls;
-    if (t < 9) nb[ls][t] = item < n ? P.nbr[list[item] * 9 + t] : -1;
-    __syncthreads();
-    if (item >= n) return;
-    const int slot = nb[ls][4];
-    const int type = P.slot_type[slot];
-    const InstParams& ip = P.inst[P.slot_inst[slot]];
+    constexpr int BB = B * B, TPR = B / 8;
     const int y = t / TPR, x0 = (t % TPR) * 8;
-    if (type != ST_INT || (P.slot_flags[slot] & (SLOTF_EDGE | SLOTF_MAILBOX | SLOTF_SOLID))) {
-        for (int i = 0; i < 8; i++)
-            fused_cell<S, C, COLL, false>(P, fin, fout, ffine, slot, type, ip, level, x0 + i, y, fhalo);
-        return;
-    }
     // all nine rows and the edge values requested before any is used
     uint4 raw[9];
     C edge[9];
@@ -1202,12 +1163,12 @@ __device__ __forceinline__ void fused_v8_task(const DevPool& P, const int* list,
         const int vy = sy < 0 ? 0 : (sy >= B ? 2 : 1);
         const int ry = sy + (vy == 0 ? B : (vy == 2 ? -B : 0));
         const size_t rowoff = (size_t)q * BB + ry * B;
-        raw[q] = ld_u4<NC>(reinterpret_cast<const uint4*>(fin + (size_t)nb[ls][vy * 3 + 1] * 9 * BB + rowoff + x0));
+        raw[q] = ld_u4<NC>(reinterpret_cast<const uint4*>(fin + (size_t)nb[vy * 3 + 1] * 9 * BB + rowoff + x0));
         edge[q] = (C)0;
         if (cx == 1 && x0 == 0)
-            edge[q] = Sto<S>::template ldr<C>(fin, (size_t)nb[ls][vy * 3 + 0] * 9 * BB + rowoff + (B - 1));
+            edge[q] = Sto<S>::template ldr<C>(fin, (size_t)nb[vy * 3 + 0] * 9 * BB + rowoff + (B - 1));
         if (cx == -1 && x0 + 8 == B)
-            edge[q] = Sto<S>::template ldr<C>(fin, (size_t)nb[ls][vy * 3 + 2] * 9 * BB + rowoff);
+            edge[q] = Sto<S>::template ldr<C>(fin, (size_t)nb[vy * 3 + 2] * 9 * BB + rowoff);
     }
     // the value each shifted plane pulls from beyond this thread's eight cells
 #pragma unroll
@@ -1221,7 +1182,6 @@ __device__ __forceinline__ void fused_v8_task(const DevPool& P, const int* list,
             if (x0 + 8 != B) edge[q] = right;
         }
     }
-    const C om = (C)1 / (C)ip.tau[level];
     unsigned ow[9][4];
     // SH: values move between the storage and the compute form by the
     // instance's shift (its nine values take registers the kernel is short
@@ -1251,6 +1211,65 @@ __device__ __forceinline__ void fused_v8_task(const DevPool& P, const int* list,
     for (int q = 0; q < 9; q++)
         *reinterpret_cast<uint4*>(fout + ((size_t)slot * 9 + q) * BB + y * B + x0) =
             make_uint4(ow[q][0], ow[q][1], ow[q][2], ow[q][3]);
+}
+// The vector sweep of the list items item0 + k stride + (0 .. SPC - 1), k = 0, 1,
+// ..., below `end` (SPC of them per thread block and pass).  What a pass needs
+// of its block -- list entry, neighbours, type, flags, instance: three dependent
+// loads -- is read one pass ahead, the list entry two, so that only the
+// populations' latency is left in a pass, and a thread block takes a contiguous
+// part of its list, whose blocks share their halo lines.  4096^2, us per step in
+// the persistent kernel / the graphs: FP32 216 / 209 -> 201 / 195 (6.0 / 6.2 TB/s,
+// 90 / 92 % of the measured copy), BF16 144 / 122 -> 123 / 119 (with a grid
+// stride the graphs' BF16 took 135).  (As a function of its own in the step
+// kernel 245 and 155; inlined it costs the D = 128 cylinder 3 %, in spills.)
+// Halo blocks and blocks on a domain side, with a mailbox or near a solid take the
+// scalar path, several cells per thread (a warp never spans two blocks).
+// The tables are kept twice, by the pass's parity: one barrier per pass, which
+// also keeps the thread block's warps on neighbouring rows.
+template <class S, class C, int B, int COLL, bool NC, bool SH>
+__device__ __forceinline__ void fused_vec_run(const DevPool& P, const int* list, int end, int item0, int stride,
+                                              const S* fin, S* fout, const S* ffine, int level, S* fhalo = nullptr) {
+    constexpr int CPT = sizeof(S) == 2 ? 8 : 4, TPS = B * B / CPT;
+    __shared__ int tab[2][STEP_MAX_THREADS / TPS][12];  // neighbours, plain (below), instance
+    const int ls = threadIdx.x / TPS, t = threadIdx.x % TPS;
+    auto entry = [&](int item) { return t < 11 && item < end ? list[item] : -1; };
+    auto read = [&](int slot) {
+        if (slot < 0) return -1;
+        if (t < 9) return P.nbr[slot * 9 + t];
+        if (t == 10) return P.slot_inst[slot];
+        return (int)(P.slot_type[slot] == ST_INT &&
+                     !(P.slot_flags[slot] & (SLOTF_EDGE | SLOTF_MAILBOX | SLOTF_SOLID)));
+    };
+    int inst = -1;
+    C om = 0;
+    if (t < 11) tab[0][ls][t] = read(entry(item0 + ls));
+    int next = entry(item0 + stride + ls);
+    __syncthreads();
+    for (int pass = 0; item0 < end; item0 += stride, pass++) {
+        const int ahead = read(next);
+        next = entry(item0 + 2 * stride + ls);
+        const int* const nb = tab[pass & 1][ls];
+        if (item0 + ls < end) {
+            const int slot = nb[4];
+            if (nb[10] != inst) {
+                inst = nb[10];
+                om = (C)1 / (C)P.inst[inst].tau[level];
+            }
+            const InstParams& ip = P.inst[inst];
+            if (!nb[9]) {
+                constexpr int TPR = B / CPT;
+                for (int i = 0; i < CPT; i++)
+                    fused_cell<S, C, COLL, false>(P, fin, fout, ffine, slot, P.slot_type[slot], ip, level,
+                                                  (t % TPR) * CPT + i, t / TPR, fhalo);
+            } else if constexpr (sizeof(S) == 2) {
+                fused_v8_cells<S, C, B, COLL, NC, SH>(P, nb, slot, om, ip, fin, fout, t);
+            } else {
+                fused_v4_cells<S, C, B, COLL, NC>(P, nb, slot, om, ip, fin, fout, t);
+            }
+        }
+        if (t < 11) tab[(pass + 1) & 1][ls][t] = ahead;
+        __syncthreads();
+    }
 }
 // ---------------------------------------------------------------------------
 // Sec. 2.4 step 2: every fine halo cell gets the post-collision populations of

@@ -1654,6 +1654,15 @@ sbot_status step_persistent(sbot_ctx* c, int most, int* ran) {
     A.bulk_rounds = c->bulk_rounds;
     A.crit_items = c->crit_items;
     A.fixed = c->groups == 1u;
+    // the lists' lengths on the device are the mirrors' (flushed before every launch)
+    A.any_vec = 0;
+    if (c->vec_min_cells >= 0 && !(P.coll & COLL_SOLID))
+        for (int i = 0; i < NLISTS; i++) {
+            const int kind = i % LK_COUNT;
+            if ((kind == LK_FUSED || kind == LK_INDEP || kind == LK_DEP) && !c->wl[i].items.empty() &&
+                (long long)c->wl[i].items.size() * c->B * c->B >= c->vec_min_cells)
+                A.any_vec = 1;
+        }
     A.max_servers = c->step_grid / 4;
     for (int l = 0; l < SBOT_MAXLEV; l++) {
         const int gl = gl_of(l + 1, l);

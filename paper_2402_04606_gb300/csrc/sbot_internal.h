@@ -250,6 +250,7 @@ struct StepArgs {
     long long spin_ns;        // longest wait for a dependency before the launch gives up (ERRB_TIMEOUT)
     int bulk_rounds;          // vector rounds per bulk task
     int crit_items;           // > 0: at most this many list items per task of a critical fused phase
+    int any_vec;              // 1: some sweep may take the vector mapping (by the host's list lengths)
     int fixed;                // 1: every task has a fixed owner (all instances have one level)
     int max_servers;          // most thread blocks set apart for one body's IBM each (more bodies: no block is)
     int body_count[SBOT_MAXLEV];  // per group, the index of its body list's length, -1 none

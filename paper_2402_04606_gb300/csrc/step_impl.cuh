@@ -140,7 +140,7 @@ __device__ int step_ntasks(const DevPool& P, const StepArgs& A, const StepPhase&
     if (n <= 0) return 0;
     switch (ph.kind) {
     case PH_FUSED: {
-        return task_shape<S, B>(A, ph, n, fused_vec<S, B>(A, ph, n, P.coll), T, grid).tasks(n);
+        return task_shape<S, B>(A, ph, n, A.any_vec && fused_vec<S, B>(A, ph, n, P.coll), T, grid).tasks(n);
     }
     case PH_C2F: {
         const int per = T >= B * B ? T / (B * B) : 1;
@@ -169,7 +169,7 @@ __device__ __forceinline__ void for_cells(int n, int i0, int k, int BB, F&& fn) 
 // and force loads remain on its path.
 // key: which task's blocks' data the shared memory holds (a thread block of a
 // launch of fixed owners runs the same task in every step, and reads them once).
-template <class S, class C, int B, int COLL, class G>
+template <class S, class C, int B, int COLL, bool VEC, class G>
 __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, int grid, int2& key,
                            G& gate) {
     __shared__ SlotMeta<C> meta[STEP_META_MAX];
@@ -180,7 +180,7 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
     const S* ffine = step_buf<S>(A, ph.ffine);
     S* fhalo = ph.fold ? step_buf<S>(A, ph.ffine) : nullptr;  // the coarse-to-fine copy rides on this sweep
     const int T = blockDim.x;
-    const bool vec = fused_vec<S, B>(A, ph, n, P.coll);
+    const bool vec = VEC && fused_vec<S, B>(A, ph, n, P.coll);
     const TaskShape sh = task_shape<S, B>(A, ph, n, vec, T, grid);
     const int per = sh.per, rounds = sh.rounds;
     if (rounds == 1 && !vec && per <= STEP_META_MAX && per <= T / 32) {
@@ -201,7 +201,7 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
         return;
     }
     if (!gate(false)) return;
-    if constexpr (B >= 16) {
+    if constexpr (B >= 16 && VEC) {
         if (vec) {
             const int i0 = local * rounds * per, end = min(n, i0 + rounds * per);
             if (sizeof(S) == 2 && (P.coll & COLL_SHIFT))
@@ -231,7 +231,7 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
 // when the launch is aborting (the task then stops).
 // An IBM task waits before its stores for the sweep of its sub-step
 // (ph.after): await() by one warp, swept() by all after a barrier (ibm_run).
-template <class S, class C, int B, int COLL, class G, class G1, class G2>
+template <class S, class C, int B, int COLL, bool VEC, class G, class G1, class G2>
 __device__ void step_task(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, int grid, int2& key,
                           unsigned char* smraw, IbmShared& sh, G& gate, G1& await, G2& swept) {
     const int* list = A.lists + ph.list_off;
@@ -240,7 +240,7 @@ __device__ void step_task(const DevPool& P, const StepArgs& A, const StepPhase& 
         return;
     }
     switch (ph.kind) {
-    case PH_FUSED: step_fused<S, C, B, COLL>(P, A, ph, local, grid, key, gate); break;
+    case PH_FUSED: step_fused<S, C, B, COLL, VEC>(P, A, ph, local, grid, key, gate); break;
     case PH_IBM:
         ibm_run<S, C, COLL>(P, list[local], step_buf<S>(A, ph.fin), step_buf<S>(A, ph.fout), ph.level, 0, 1, ph.arg,
                             smraw, sh, gate, await, swept);
@@ -358,7 +358,11 @@ __device__ bool wait_until(const DevPool& P, const StepArgs& A, R&& ready) {
     }
 }
 
-template <class S, class C, int B, int COLL>
+// VEC: some sweep of the launch takes the vector mapping (StepArgs::any_vec).  A
+// kernel without it: the vector sweep's registers make the rest spill
+// (immersed cylinder in a cavity 36.2 -> 32.4 us per step without it, D = 40
+// cylinder 50.5 -> 49.8).
+template <class S, class C, int B, int COLL, bool VEC>
 __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_step(const __grid_constant__ DevPool P, const __grid_constant__ StepArgs A) {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ IbmShared sh;
@@ -594,7 +598,7 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
             if ((threadIdx.x & 31) == 0 && !ok) s_go = 0;
         };
         auto swept = [&]() -> bool { return s_go != 0; };
-        step_task<S, C, B, COLL>(P, A, A.ph[s_phase], s_local, workers, s_key, smraw, sh, gate, await, swept);
+        step_task<S, C, B, COLL, VEC>(P, A, A.ph[s_phase], s_local, workers, s_key, smraw, sh, gate, await, swept);
         __syncthreads();  // the task's writes, then its count (a release: the
                           // barrier orders every thread's writes before it)
         if (threadIdx.x == 0 && s_go) {
@@ -632,7 +636,7 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
 
 template <class S, class C, int B, int COLL>
 cudaError_t launch_step_k(const DevPool& P, const StepArgs& A, int grid, int threads, size_t smem, cudaStream_t s) {
-    auto kern = k_step<S, C, B, COLL>;
+    auto kern = B >= 16 && A.any_vec ? k_step<S, C, B, COLL, (B >= 16)> : k_step<S, C, B, COLL, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -650,7 +654,7 @@ cudaError_t launch_step_k(const DevPool& P, const StepArgs& A, int grid, int thr
 
 template <class S, class C, int B, int COLL>
 int occupancy_k(int threads, size_t smem, size_t* static_smem) {
-    auto kern = k_step<S, C, B, COLL>;
+    auto kern = k_step<S, C, B, COLL, (B >= 16)>;  // the larger of the two in registers and shared memory
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return 0;
     if (static_smem) *static_smem = fa.sharedSizeBytes;

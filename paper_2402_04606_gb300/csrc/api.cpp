@@ -47,8 +47,9 @@ struct HostBody {
 //   GF     fine-side halo blocks (coarse-to-fine copy)
 //   GC     coarse-side mailbox blocks (no launch of their own: the coarse
 //          pull merges the fine values; the list keeps their membership)
-//   INDEP  fused blocks that need no mailbox and hold no cell a body forces
-//   DEP    the other interior blocks
+//   INDEP  fused blocks that need no mailbox and have no cell within one cell of
+//          the stencils of a body
+//   DEP    the others
 //   IBM    instances whose finest level this is
 // Lists are unordered: every block of a launch is independent of the others.
 enum { LK_FUSED = 0, LK_GF, LK_GC, LK_INDEP, LK_DEP, LK_IBM, LK_COUNT };
@@ -490,7 +491,7 @@ void list_remove(sbot_ctx* c, int gl, int k, int id, int units) {
 // the lists a slot of `type` belongs to
 uint8_t kinds_of(int type, bool dep) {
     if (type == ST_INT) return (uint8_t)((1 << LK_FUSED) | (1 << (dep ? LK_DEP : LK_INDEP)));
-    if (type == ST_GF) return (uint8_t)((1 << LK_FUSED) | (1 << LK_GF) | (1 << LK_INDEP));
+    if (type == ST_GF) return (uint8_t)((1 << LK_FUSED) | (1 << LK_GF) | (1 << (dep ? LK_DEP : LK_INDEP)));
     if (type == ST_GC) return (uint8_t)(1 << LK_GC);
     return 0;
 }
@@ -1056,10 +1057,13 @@ sbot_status build_topology(sbot_ctx* c, int ii, long long n, bool transfer) {
     }
     I.ip.latmap = I.d_latmap;
     if (first) TRY(upload(c, c->d_ip + ii, &I.ip, sizeof(InstParams)));
-    // interior blocks in the lists of their own: those with a mailbox neighbour
-    // (coarse side of an interface), which wait for the finer level, and on the
-    // finest level those a body may force (every finest block for a moving body;
-    // the stencil box for a static one), which the IBM waits for
+    // blocks in the lists of their own: those with a mailbox neighbour (coarse side
+    // of an interface), which wait for the finer level, and on the finest level
+    // those a body may force (every interior block for a moving body) or that pull
+    // from, or overwrite, what the IBM of a static body writes and pulls: every
+    // interior or halo block with a cell in the box of its stencils and the cells
+    // next to them, also across a periodic side.  (The others' sweep does not wait
+    // for the IBM in the persistent kernel.)
     int bx0 = 1 << 30, by0 = 1 << 30, bx1 = -(1 << 30), by1 = -(1 << 30);
     const bool static_body = I.has_body && I.body.motion == 0;
     if (static_body) {
@@ -1068,13 +1072,23 @@ sbot_status build_topology(sbot_ctx* c, int ii, long long n, bool transfer) {
             double qx = I.body.qx[j] - I.body.pivot[0], qy = I.body.qy[j] - I.body.pivot[1];
             double rx = I.body.x0[0] + I.body.pivot[0] + cs * qx - sn * qy;
             double ry = I.body.x0[1] + I.body.pivot[1] + sn * qx + cs * qy;
-            int i0 = (int)std::floor(rx - 0.5) - 1, j0 = (int)std::floor(ry - 0.5) - 1;
-            bx0 = std::min(bx0, i0 - 1);
-            by0 = std::min(by0, j0 - 1);
-            bx1 = std::max(bx1, i0 + 4);
-            by1 = std::max(by1, j0 + 4);
+            // (the kernel's marker may differ in its last bits)
+            bx0 = std::min(bx0, (int)std::floor(rx - 0.5 - 1e-6) - 2);
+            by0 = std::min(by0, (int)std::floor(ry - 0.5 - 1e-6) - 2);
+            bx1 = std::max(bx1, (int)std::floor(rx - 0.5 + 1e-6) + 3);
+            by1 = std::max(by1, (int)std::floor(ry - 0.5 + 1e-6) + 3);
         }
     }
+    const int nxf = I.d.nx0 << (I.m - 1), nyf = I.d.ny0 << (I.m - 1);
+    auto meets_stencils = [&](const PlannedBlock& pb) {
+        bool mx = false, my = false;
+        for (int k = -1; k <= 1; k++) {
+            const int x0 = pb.bx * c->B + k * nxf, y0 = pb.by * c->B + k * nyf;
+            mx |= (k == 0 || px) && x0 <= bx1 && bx0 < x0 + c->B;
+            my |= (k == 0 || py) && y0 <= by1 && by0 < y0 + c->B;
+        }
+        return mx && my;
+    };
     std::vector<int> ints;
     I.ip.solid_blocks = 0;
     for (int l = 0; l < I.m; l++) {
@@ -1096,12 +1110,10 @@ sbot_status build_topology(sbot_ctx* c, int ii, long long n, bool transfer) {
                     set_tab(c, c->h_flags, A_FLAGS, sl, c->h_flags[sl] | (int)SLOTF_SOLID);
                     set_tab(c, c->h_parent, A_PARENT, sl, I.ip.solid_blocks++);  // its entry in the links' table
                 }
-                if (l == I.m - 1 && I.has_body) {
-                    int x0 = pb.bx * c->B, y0 = pb.by * c->B;
-                    dep = dep || !static_body || (x0 <= bx1 && bx0 < x0 + c->B && y0 <= by1 && by0 < y0 + c->B);
-                }
+                if (l == I.m - 1 && I.has_body) dep = dep || !static_body || meets_stencils(pb);
             } else {
                 units = popcount_mask(pb.mask);
+                if (l == I.m - 1 && static_body) dep = pb.type == ST_GF && meets_stencils(pb);
             }
             set_membership(c, sl, gl_of(I.m, l), kinds_of(pb.type, dep), units);
         }
@@ -1434,7 +1446,7 @@ struct PhaseEmit {
         const int forced = l == g ? last_ibm : -1;  // the level's previous IBM wrote the cells this sweep pulls
         int A = -1, Bp;
         if (fork) {
-            // (blocks away from a static body's stencils neither pull nor overwrite a cell that the IBM touches)
+            // (static bodies: the list's blocks neither pull nor overwrite a cell that the IBM touches, build_topology)
             A = add(PH_FUSED, l, gl, LK_INDEP, {lastA[l], lastB[l], c2, moving ? forced : -1}, cur, nxt, fine);
             Bp = add(PH_FUSED, l, gl, LK_DEP, {lastA[l], lastB[l], c2, forced, fa, fb}, cur, nxt, fine,
                      l < g ? 1 : 0);  // next to the finer region: one cell per thread

@@ -1,0 +1,86 @@
+"""Sweeps beside the IBM of a static body: a sweep that pulls from, or
+overwrites, the cells the IBM writes and pulls waits for it, wherever its
+blocks lie.
+
+Stencils whose last (or first) cell lies on a periodic side (the blocks across
+the side pull the forced cells), in a corner of two periodic sides, and stencils
+that reach the outermost interior cells of the finest level (the halo blocks
+beside it stream from forced cells, and the coarse level merges them): the
+persistent kernel equals the per-phase graphs bit for bit, and in FP64 both
+equal the oracle to the parity tolerance.
+"""
+import numpy as np
+import pytest
+
+from paper_2402_04606_gb300 import workloads as wl
+from tests.helpers import init_oracle, initial_fields, oracle_from_spec, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+P = wl.BC_PERIODIC
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2402_04606_gb300 import build
+
+    build.build()
+
+
+def body(x0):
+    return wl.BodySpec(a=5.0, b=5.0, n_markers=31, x0=x0)
+
+
+def seam(x0, block, storage):
+    """one level: a circle whose stencils end on a periodic side"""
+    return wl.DomainSpec("seam", 64, 64, levels=1, block=block, bc=(P,) * 4, tau_finest=0.6, u_in=(0.05, 0.02),
+                         storage=storage, body=body(x0))
+
+
+def rim(x0, block, storage):
+    """two levels, the finer one from cell 32 to 79 (blocks of 8) or 95 (of 16): a circle at its rim"""
+    top = 79.0 if block == 8 else 95.0
+    return wl.DomainSpec("rim", 64, 64, levels=2, block=block, bc=(P,) * 4, tau_finest=0.6, u_in=(0.05, 0.02),
+                         storage=storage, boxes=[(1, 33.0, 33.0, top, top)], body=body(x0))
+
+
+LAYOUTS = [(seam, (57.0, 32.0)), (seam, (32.0, 57.0)), (seam, (57.0, 57.0)), (seam, (7.6, 32.0)),
+           (rim, (39.0, 56.0)), (rim, (56.0, 39.0)), (rim, (39.0, 39.0))]
+
+
+def run(spec, persistent, steps, vec):
+    from paper_2402_04606_gb300.native import TUNE_PERSISTENT, TUNE_VECTOR_MIN_CELLS, Domain
+
+    g = Domain(spec)
+    g.set_tuning(TUNE_PERSISTENT, persistent)
+    g.set_tuning(TUNE_VECTOR_MIN_CELLS, vec)
+    for l in range(spec.levels):
+        g.set_fields(l, *initial_fields(spec, l))
+    g.step(steps)
+    out = [g.populations(l) for l in range(spec.levels)], g.forces()
+    g.close()
+    return out
+
+
+@pytest.mark.parametrize("block,storage,vec", [(8, wl.F64, -1), (8, wl.F32, -1), (16, wl.F64, 0), (16, wl.F32, 0)])
+@pytest.mark.parametrize("make,x0", LAYOUTS)
+def test_sweep_waits_for_the_ibm_whose_cells_it_touches(make, x0, block, storage, vec):
+    spec, steps = make(x0, block, storage), 33
+    pops, forces = run(spec, 1, steps, vec)
+    gp, gf = run(spec, 0, steps, vec)
+    for a, b in zip(pops, gp):
+        assert np.array_equal(a, b)
+    assert np.array_equal(forces, gf)
+    if storage != wl.F64:
+        return
+    o = init_oracle(oracle_from_spec(spec), spec)
+    o.step(steps)
+    for l in range(spec.levels):
+        m = o.types(l) == 1
+        assert rel_l2(pops[l][:, m], o.populations(l)[:, m]) <= 1e-12
+    fo = o.forces()
+    np.testing.assert_allclose(forces[:, :2], fo[:, :2], rtol=1e-10, atol=1e-11 * np.abs(fo[:, :2]).max())

@@ -168,7 +168,9 @@ __device__ __forceinline__ void for_cells(int n, int i0, int k, int BB, F&& fn) 
 // phases it depends on have finished: after the gate only the population
 // and force loads remain on its path.
 // key: which task's blocks' data the shared memory holds (a thread block of a
-// launch of fixed owners runs the same task in every step, and reads them once).
+// launch of fixed owners runs the same task in every step, and reads them once;
+// there a list is cut the same way in every phase, which elsewhere it is not: a
+// level-0 list is bulk in the first step and critical in the others).
 template <class S, class C, int B, int COLL, bool VEC, class G>
 __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, int grid, int2& key,
                            G& gate) {
@@ -188,10 +190,10 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
         // its cells: those of its items, or a part of one item's
         const int len = sh.parts > 1 ? B * B / sh.parts : (ne - i0) * B * B;
         const int c0 = sh.parts > 1 ? (local - i0 * sh.parts) * len : 0;
-        const bool held = key.x == ph.list_off && key.y == local;
+        const bool held = A.fixed && key.x == ph.list_off && key.y == local;
         if (!held && i0 + w < ne) load_meta<C>(P, list[i0 + w], ph.level, meta[w]);
         if (!gate(true)) return;
-        if (threadIdx.x == 0) key = make_int2(ph.list_off, local);
+        if (A.fixed && threadIdx.x == 0) key = make_int2(ph.list_off, local);
         for (int c = c0 + threadIdx.x; c < c0 + len; c += T) {
             const SlotMeta<C>& m = meta[c / (B * B)];
             const int cell = c % (B * B);

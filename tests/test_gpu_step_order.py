@@ -84,3 +84,30 @@ def test_sweep_waits_for_the_ibm_whose_cells_it_touches(make, x0, block, storage
         assert rel_l2(pops[l][:, m], o.populations(l)[:, m]) <= 1e-12
     fo = o.forces()
     np.testing.assert_allclose(forces[:, :2], fo[:, :2], rtol=1e-10, atol=1e-11 * np.abs(fo[:, :2]).max())
+
+
+@pytest.mark.parametrize("threads,rounds,crit", [(768, 8, 1), (768, 8, 2), (256, 8, 1), (768, 1, 0), (256, 1, 0),
+                                                 (768, 1, 2)])
+@pytest.mark.parametrize("make", [
+    lambda: wl.cylinder(D=10, levels=3, block=8, storage=wl.F32),                              # 50 level-0 blocks
+    lambda: wl.cylinder(D=20, levels=2, block=16, storage=wl.F32, n_markers=63),               # 190
+    lambda: wl.cylinder(D=40, levels=2, block=8, storage=wl.F32)], ids=["8 short", "16", "8 long"])  # 2850
+def test_task_sizes_do_not_change_results(make, threads, rounds, crit):
+    """a list that is cut differently in the first step (bulk tasks) and in the others, several steps per launch:
+    each task sweeps its own blocks, whatever its thread block swept before under the same task number"""
+    from paper_2402_04606_gb300 import native as nv
+
+    spec, res = make(), []
+    for knobs in ((threads, rounds, crit), (0, 8, 0)):
+        g = nv.Domain(spec)
+        g.set_tuning(nv.TUNE_VECTOR_MIN_CELLS, -1)
+        for what, v in zip((nv.TUNE_STEP_THREADS, nv.TUNE_BULK_ROUNDS, nv.TUNE_CRIT_BLOCKS), knobs):
+            g.set_tuning(what, v)
+        for l in range(spec.levels):
+            g.set_fields(l, *initial_fields(spec, l))
+        g.step(64)
+        res.append(([g.populations(l) for l in range(spec.levels)], g.forces()))
+        g.close()
+    for a, b in zip(res[0][0], res[1][0]):
+        assert np.array_equal(a, b)
+    assert np.array_equal(res[0][1], res[1][1])

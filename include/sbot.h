@@ -431,7 +431,8 @@ sbot_status sbot_batch_create(int max_instances, int block, int storage, int64_t
  * joins the next sbot_step.  *slot receives its index (the lowest free one).
  * The budget check counts two population buffers for every block the
  * instance needs at time 0 (1.5 times as many when a moving body re-tags),
- * its body buffers and lattice maps, against what the live instances hold.
+ * its body buffers, the table of its solid and its lattice maps, against what
+ * the live instances hold.
  * Errors: SBOT_ERR_ARG, SBOT_ERR_OOM (no free slot, over the budget, or a
  * failed allocation; the batch is unchanged), SBOT_ERR_STATE (refinement
  * reaches a non-periodic side). */

@@ -843,6 +843,21 @@ bool solid_near_block(const InstParams& ip, int x0, int y0, int B) {
     return x0 < b[2] && b[0] < x0 + B && y0 < b[3] && b[1] < y0 + B;
 }
 
+// every cell of the block lies inside the solid (by a little: the kernels' own
+// test of a cell may differ in its last bits); the solid and the block are convex
+bool solid_fills_block(const InstParams& ip, int x0, int y0, int B) {
+    if (ip.solid == 2) return y0 + B - 0.5 < ip.sol[0] - 1e-6;
+    double r = 0;
+    for (int k = 0; k < 4; k++)
+        r = std::max(r, std::hypot(x0 + (k & 1 ? B - 0.5 : 0.5) - ip.sol[0], y0 + (k & 2 ? B - 0.5 : 0.5) - ip.sol[1]));
+    return ip.solid == 1 && r < ip.sol[2] - 1e-6;
+}
+
+// the block has cells whose links may meet the solid: an entry in the links' table
+bool solid_has_links(const InstParams& ip, int x0, int y0, int B) {
+    return solid_near_block(ip, x0, y0, B) && !solid_fills_block(ip, x0, y0, B);
+}
+
 // every cell within two cells of a solid cell is a finest interior cell (or
 // solid) and inside the domain (a circle), under a static refinement
 bool solid_clear(const InstParams& ip, int m, const BlockStates& bs, int B, bool px, bool py) {
@@ -1108,7 +1123,8 @@ sbot_status build_topology(sbot_ctx* c, int ii, long long n, bool transfer) {
                 if (dep) set_tab(c, c->h_flags, A_FLAGS, sl, c->h_flags[sl] | (int)SLOTF_MAILBOX);
                 if (l == I.m - 1 && solid_near_block(I.ip, pb.bx * c->B, pb.by * c->B, c->B)) {
                     set_tab(c, c->h_flags, A_FLAGS, sl, c->h_flags[sl] | (int)SLOTF_SOLID);
-                    set_tab(c, c->h_parent, A_PARENT, sl, I.ip.solid_blocks++);  // its entry in the links' table
+                    if (solid_has_links(I.ip, pb.bx * c->B, pb.by * c->B, c->B))
+                        set_tab(c, c->h_parent, A_PARENT, sl, I.ip.solid_blocks++);  // its entry in the links' table
                 }
                 if (l == I.m - 1 && I.has_body) dep = dep || !static_body || meets_stencils(pb);
             } else {
@@ -1130,12 +1146,11 @@ sbot_status build_topology(sbot_ctx* c, int ii, long long n, bool transfer) {
         I.int_cap = ncap;
     }
     TRY(upload(c, I.d_int, ints.data(), ints.size() * sizeof(int)));
-    if (I.ip.solid_blocks > 0) {  // the links' table (filled once the slot tables are written, by admit)
-        CK(cudaStreamSynchronize(c->s));
-        dfree(I.d_solid);
-        I.d_solid = nullptr;
-        CK(cudaMalloc(&I.d_solid, solid_table_bytes(c->storage, I.ip.solid_blocks, c->B * c->B)));
+    if (I.ip.solid_blocks > 0 && !I.d_solid) {  // the links' table (filled once the slot tables are written, by admit)
+        const size_t bytes = solid_table_bytes(c->storage, I.ip.solid_blocks, c->B * c->B);
+        CK(cudaMalloc(&I.d_solid, bytes));
         I.ip.solid_tab = I.d_solid;
+        I.extra_bytes += (long long)bytes;  // (check_budget has counted it)
         TRY(upload(c, c->d_ip + ii, &I.ip, sizeof(InstParams)));
     }
     I.ts = ts;
@@ -2099,7 +2114,7 @@ sbot_status create_ctx(int max_instances, int block, int storage, long long budg
 
 // Admission by device footprint: the slots the instance needs at its first
 // coarse step (half as many again when its refined region moves), its body
-// buffers and its lattice maps must fit next to what the live instances hold.
+// buffers, its solid's table and its lattice maps must fit next to what the live instances hold.
 sbot_status check_budget(sbot_ctx* c, const Inst& I) {
     if (c->budget <= 0) return SBOT_OK;
     TopoSpec ts = topo_spec(I, c->B);
@@ -2109,10 +2124,13 @@ sbot_status check_budget(sbot_ctx* c, const Inst& I) {
     if (!plan_blocks(ts, bs, &why)) return fail(c, SBOT_ERR_STATE, why);
     std::vector<PlannedBlock> pbs;
     plan_slots(ts, bs, pbs);
-    long long lat = 0;
+    long long lat = 0, linked = 0;
     for (int l = 0; l < I.m; l++) lat += (long long)bs.nbx[l] * bs.nby[l] * 4;
+    for (const PlannedBlock& pb : pbs)
+        linked += pb.type == ST_INT && pb.level == I.m - 1 && solid_has_links(I.ip, pb.bx * c->B, pb.by * c->B, c->B);
     double envelope = (I.d.retag && I.has_body) ? 1.5 : 1.0;
-    long long need = (long long)((double)pbs.size() * envelope) * 2 * (long long)slot_bytes(c) + I.extra_bytes + lat;
+    long long need = (long long)((double)pbs.size() * envelope) * 2 * (long long)slot_bytes(c) + I.extra_bytes + lat +
+                     (long long)solid_table_bytes(c->storage, (int)linked, c->B * c->B);
     if (bytes_in_use(c) + need > c->budget)
         return fail(c, SBOT_ERR_OOM, "admission refused: the instance does not fit the device-memory budget");
     return SBOT_OK;

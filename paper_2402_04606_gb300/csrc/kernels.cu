@@ -126,8 +126,9 @@ __global__ void __launch_bounds__(1024) k_solid_table(const __grid_constant__ De
                                                       void* tab, int blocks, int level) {
     const int slot = list[blockIdx.x], B = P.B, BB = B * B, cell = threadIdx.x;
     if ((int)blockIdx.x >= n || !(P.slot_flags[slot] & SLOTF_SOLID)) return;
-    const size_t blk = (size_t)P.slot_parent[slot];
-    if (blk >= (size_t)blocks) return;
+    const int entry = P.slot_parent[slot];
+    if (entry < 0 || entry >= blocks) return;  // (the solid fills the block)
+    const size_t blk = (size_t)entry;
     C* const coef = (C*)tab;
     unsigned* const word = (unsigned*)(coef + (size_t)blocks * BB * 16);
     solid_fill<C>(P.inst[P.slot_inst[slot]], level, P.slot_ox[slot] + cell % B, P.slot_oy[slot] + cell / B, cell, BB,

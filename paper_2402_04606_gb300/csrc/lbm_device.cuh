@@ -775,7 +775,9 @@ __device__ __noinline__ bool solid_links(const DevPool& P, const S* fin, int slo
 // does the refinement around them): per cell of a block near a solid one word --
 // bit q: the source of direction q is solid; bit 9 + q: its t < 1/2 form applies;
 // bit 20: the cell is solid -- and per direction the form's two factors in the
-// compute type.  A block's entry is the index its slot_parent holds.
+// compute type.  A block's entry is the index its slot_parent holds; a block that
+// the solid fills has none (-1).  68 bytes per cell (132 in FP64), about a
+// block's populations once more, so only for blocks at the solid's surface.
 #define SOLID_CELL (1u << 20)
 template <class C>
 struct SolidTab {
@@ -879,6 +881,7 @@ __device__ __forceinline__ void fused_cell(const DevPool& P, M mt, const S* fin,
     const C* coef = nullptr;
     if constexpr (SOLID) {
         if (flags & SLOTF_SOLID) {
+            if (mt.parent() < 0) return;  // inside the solid: left as it is
             const SolidTab<C> tab(ip.solid_tab, ip.solid_blocks, BB);
             const size_t blk = (size_t)mt.parent();
             links = tab.word[blk * BB + cell];

@@ -1830,12 +1830,21 @@ sbot_status reset_state(sbot_ctx* c, int ii) {
     return SBOT_OK;
 }
 
+long long bytes_in_use(const sbot_ctx* c) {
+    long long used = (long long)(c->cap - (long long)c->free_slots.size()) * 2 * (long long)slot_bytes(c);
+    for (auto& I : c->inst)
+        if (I.live) used += I.extra_bytes + I.latmap_n * 4 + I.int_cap * 4;
+    return used;
+}
+
 // Dense export of a level of instance I: mode 0 populations, mode 1 fields, the
 // `planes` planes to out[i] (nullptr: left out), `per` planes each.  The copies
 // go straight to the caller's arrays (through an array of its own and one
 // memcpy per plane, 4096^2 fields took 59 ms, now 20), and a device buffer of
 // up to EXPORT_KEPT bytes is kept for the next call: cudaMalloc and cudaFree
-// wait for the whole device.
+// wait for the whole device.  In a context with a memory budget it is kept only
+// beside instances that leave room for it, and goes before an admission is refused
+// for its sake (check_budget).
 constexpr size_t EXPORT_KEPT = size_t(64) << 20;
 sbot_status export_level(sbot_ctx* c, Inst& I, int level, int mode, double* const* out, int n_out) {
     int nx = I.d.nx0 << level, ny = I.d.ny0 << level;
@@ -1843,8 +1852,10 @@ sbot_status export_level(sbot_ctx* c, Inst& I, int level, int mode, double* cons
     int planes = mode == 0 ? 9 : 3;
     const size_t bytes = (size_t)planes * plane * sizeof(double), part = bytes / n_out;
     double* d = nullptr;
-    const bool keep = bytes <= EXPORT_KEPT;
-    if (keep && c->export_cap >= bytes) {
+    const bool held = c->export_cap >= bytes;
+    const bool keep = held || (bytes <= EXPORT_KEPT &&
+                               (c->budget <= 0 || bytes_in_use(c) + (long long)bytes <= c->budget));
+    if (held) {
         d = c->d_export;
     } else {
         if (keep) {
@@ -1921,13 +1932,6 @@ void free_inst_device(Inst& I) {
     I.d_hist = nullptr;
     I.latmap_n = 0;
     I.int_cap = 0;
-}
-
-long long bytes_in_use(const sbot_ctx* c) {
-    long long used = (long long)(c->cap - (long long)c->free_slots.size()) * 2 * (long long)slot_bytes(c);
-    for (auto& I : c->inst)
-        if (I.live) used += I.extra_bytes + I.latmap_n * 4 + I.int_cap * 4;
-    return used;
 }
 
 // instance ii from its descriptions (no slots yet)
@@ -2131,6 +2135,12 @@ sbot_status check_budget(sbot_ctx* c, const Inst& I) {
     double envelope = (I.d.retag && I.has_body) ? 1.5 : 1.0;
     long long need = (long long)((double)pbs.size() * envelope) * 2 * (long long)slot_bytes(c) + I.extra_bytes + lat +
                      (long long)solid_table_bytes(c->storage, (int)linked, c->B * c->B);
+    if (c->d_export && bytes_in_use(c) + need + (long long)c->export_cap > c->budget) {
+        CK(cudaStreamSynchronize(c->s));
+        dfree(c->d_export);
+        c->d_export = nullptr;
+        c->export_cap = 0;
+    }
     if (bytes_in_use(c) + need > c->budget)
         return fail(c, SBOT_ERR_OOM, "admission refused: the instance does not fit the device-memory budget");
     return SBOT_OK;

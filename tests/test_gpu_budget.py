@@ -1,6 +1,7 @@
 """Device memory that an instance or a context holds beside its populations:
 the table of a solid's links is part of the admission budget, and is kept only
-for the blocks at the solid's surface.
+for the blocks at the solid's surface; the device buffer of a read-out is kept
+only where the budget leaves room for it.
 """
 import numpy as np
 import pytest
@@ -69,3 +70,35 @@ def test_solid_table_is_in_the_budget():
     with pytest.raises(SbotError) as e:
         admitted_bytes(half, bytes_ - lists - 1)
     assert e.value.status == ERR_OOM
+
+
+def test_kept_read_out_buffer_stays_inside_the_budget():
+    import torch
+
+    from paper_2402_04606_gb300.native import Batch
+
+    spec = wl.tgv(n=1024, block=16, storage=wl.F32)
+    buffer = 3 * 8 * 1024 * 1024  # what a read of its fields needs on the device
+    one = Batch(1, block=16, storage=wl.F32)  # (also loads the kernels)
+    i = one.admit(spec)
+    want = i.fields(0)
+    bytes_ = one.info()["bytes"]
+    one.close()
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    b = Batch(1, block=16, storage=wl.F32, budget_bytes=bytes_ + buffer // 2)  # no room beside the instance
+    i, before = b.admit(spec), free()
+    got = i.fields(0)
+    assert before - free() < buffer // 4
+    b.close()
+    b = Batch(2, block=16, storage=wl.F32, budget_bytes=2 * bytes_ + buffer // 2)  # room until the second one comes
+    i = b.admit(spec)
+    i.fields(0)
+    j = b.admit(spec)
+    again = j.fields(0)
+    b.close()
+    for x, y, z in zip(want, got, again):
+        assert np.array_equal(x, y) and np.array_equal(x, z)

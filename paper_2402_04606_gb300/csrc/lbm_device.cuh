@@ -546,6 +546,8 @@ __device__ __forceinline__ void load_meta(const DevPool& P, int slot, int level,
             const int k = e / 9, q = e % 9;
             m.wall[k][q] = (C)wall_gain(ip, k, q);
         }
+    } else if (lane < 4) {
+        m.kind[lane] = -1;  // a missing neighbour is then an error (ERRB_NOSOURCE), not a side
     }
     if (lane < 9) {
         const int ns = P.nbr[slot * 9 + lane];

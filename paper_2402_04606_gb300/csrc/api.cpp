@@ -1876,13 +1876,16 @@ sbot_status export_level(sbot_ctx* c, Inst& I, int level, int mode, double* cons
                       I.coarse_step == 0 ? 1 : 0, nx, d, plane, mode, c->s);
         e = cudaGetLastError();
     }
-    for (int i = 0; i < n_out && e == cudaSuccess; i++)
+    // (an error leaves the caller's arrays as they are)
+    const sbot_status st = e == cudaSuccess ? check_device_error(c) : SBOT_OK;
+    for (int i = 0; i < n_out && e == cudaSuccess && st == SBOT_OK; i++)
         if (out[i]) e = cudaMemcpyAsync(out[i], (const char*)d + i * part, part, cudaMemcpyDeviceToHost, c->s);
     cudaError_t e2 = cudaStreamSynchronize(c->s);
     if (!keep) dfree(d);
+    TRY(st);
     CK(e);
     CK(e2);
-    return check_device_error(c);
+    return SBOT_OK;
 }
 
 sbot_status validate_desc(const sbot_domain_desc* d, std::string& why) {

@@ -172,8 +172,6 @@ struct sbot_ctx {
     double* d_out3 = nullptr;
     double* d_export = nullptr;  // kept dense export buffer (export_level)
     size_t export_cap = 0;       // bytes
-    char* pin = nullptr;         // pinned memory for small read-outs (at most twice a full force history)
-    size_t pin_cap = 0;
     // concurrency: a stream per group, and per (group, level) a side stream
     // for the blocks that need not wait (created when the group first appears)
     cudaStream_t gstream[SBOT_MAXLEV] = {};
@@ -314,6 +312,17 @@ sbot_status arena_put(sbot_ctx* c, const void* src, size_t bytes, const char** o
     a.used = at + bytes;
     *out = a.host + at;
     return SBOT_OK;
+}
+
+// `bytes` of pinned memory for a copy to the host that is waited for before
+// anything else is staged: what the arenas leave unused (admission has made one, of
+// 1 MB at least); nullptr when neither has as much
+char* staging_room(sbot_ctx* c, size_t bytes) {
+    for (Arena& a : c->arena) {
+        const size_t at = (a.used + 15) & ~size_t(15);
+        if (a.host && at + bytes <= a.cap) return a.host + at;
+    }
+    return nullptr;
 }
 
 // asynchronous host-to-device copy through the staging memory
@@ -2522,18 +2531,13 @@ sbot_status sbot_get_forces(sbot_ctx_t c, double* fx, double* fy, double* mz, in
     long long avail = upto - I->forces_read;
     const int cnt = avail > SBOT_HIST_CAP ? 0 : (int)std::min<long long>(avail, *n_inout);
     // the error word and the entries in one wait, through pinned memory (three
-    // waits and pageable copies took 20 us a call)
+    // waits and pageable copies took 20 us a call; pinned memory of its own, 70 to 110
+    // us at a context's first call)
     const size_t need = 16 + (size_t)3 * cnt * sizeof(double);
-    if (need > c->pin_cap) {
-        if (c->pin) cudaFreeHost(c->pin);
-        c->pin = nullptr;
-        c->pin_cap = 0;
-        const size_t ncap = std::max<size_t>(2 * need, size_t(1) << 16);
-        CK(cudaHostAlloc((void**)&c->pin, ncap, cudaHostAllocDefault));
-        c->pin_cap = ncap;
-    }
-    int* const err = (int*)c->pin;
-    double* const h = (double*)(c->pin + 16);
+    char* const pin = staging_room(c, need);
+    std::vector<double> own(pin ? 0 : 2 + (size_t)3 * cnt);
+    int* const err = pin ? (int*)pin : (int*)own.data();
+    double* const h = pin ? (double*)(pin + 16) : own.data() + 2;
     // the ring holds entry k at k mod capacity: at most two contiguous pieces
     const long long k0 = I->forces_read % SBOT_HIST_CAP;
     const long long first = std::min<long long>(cnt, SBOT_HIST_CAP - k0);
@@ -2807,7 +2811,6 @@ sbot_status sbot_destroy(sbot_ctx_t c) {
                   c->d_counts, c->d_jobs,  c->d_out3,  c->d_one,    c->d_partials, c->d_recs,
                   c->d_ph[0],  c->d_ph[1], c->d_ph[2], c->d_ph[3], c->d_ctl, c->d_trace, c->d_export};
     for (void* p : ps) dfree(p);
-    if (c->pin) cudaFreeHost(c->pin);
     for (auto& I : c->inst) free_inst_device(I);
     for (int g = 0; g < 2; g++) drop_graph(c, g);
     for (int i = 0; i < 2; i++) {

@@ -44,3 +44,25 @@ def test_error_leaves_the_arrays(call):
     assert (out == -7.0).all()
     assert read(g.h, 0, *args, C.byref(n)) == OK and (out != -7.0).all()
     g.close()
+
+
+@pytest.mark.parametrize("steps", [1, 700, 16000])  # 4, 2800 and 64000 entries: the last exceed the staging memory
+def test_long_and_short_force_reads_agree(steps):
+    from paper_2402_04606_gb300.native import Domain
+
+    spec = wl.cylinder(D=10, levels=3, block=8, storage=wl.F32, re=100.0)
+    whole, parts = [], []
+    for parts_of, out in ((steps, whole), (max(1, steps // 7), parts)):
+        g = Domain(spec)
+        for l in range(spec.levels):
+            g.set_fields(l, *initial_fields(spec, l))
+        left = steps
+        while left:
+            n = min(left, parts_of)
+            g.step(n)
+            out.append(g.forces())
+            left -= n
+        assert g.forces().shape == (0, 3)
+        g.close()
+    a, b = np.concatenate(whole), np.concatenate(parts)
+    assert a.shape == (4 * steps, 3) and np.array_equal(a, b) and np.abs(a[:, 0]).min() > 0

@@ -36,9 +36,9 @@
 // decision, so a broken schedule returns an error instead of hanging the
 // device.  Two exceptions to this hand-out, explained where they begin below:
 // the IBM servers (an IBM task waits once more, before its stores, for its
-// sub-step's sweep; that sweep is ready whenever the IBM is and comes before it
-// in the order, so where a thread block takes both kinds the sweep's tasks are
-// all taken first), and the fixed owners of single-level launches.
+// sub-step's sweep, which comes before it in the order; where a thread block
+// takes both kinds, an IBM task is handed out only after all of that sweep's),
+// and the fixed owners of single-level launches.
 //
 // Reads of buffers that other thread blocks wrote earlier in the launch use
 // plain loads (no read-only cache path): the acquire fence after the
@@ -305,7 +305,7 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 // The dependencies of every phase, copied to shared memory at the start of
 // the launch (the phase table does not change during it).
 struct StepDeps {
-    int n[STEP_MAX_PHASES];
+    int n[STEP_MAX_PHASES];  // their number; from bit 8 on, 1 + the phase awaited before the stores (StepPhase::after)
     unsigned short d[STEP_MAX_PHASES][8];
 };
 
@@ -313,7 +313,7 @@ struct StepDeps {
 // Relaxed loads, issued together: a screen; a yes is confirmed by
 // deps_acquire before the task runs.
 __device__ __forceinline__ bool deps_screen(const StepArgs& A, const StepDeps& D, int q, const int* ntask) {
-    const int nd = D.n[q];
+    const int nd = D.n[q] & 255;
     bool ok = true;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
@@ -331,7 +331,7 @@ __device__ __forceinline__ bool deps_screen(const StepArgs& A, const StepDeps& D
 __device__ __forceinline__ bool deps_acquire(const StepArgs& A, const StepDeps& D, int q, const int* ntask) {
     const int lane = threadIdx.x & 31;
     bool ok = true;
-    if (lane < D.n[q]) {
+    if (lane < (D.n[q] & 255)) {
         const int d = D.d[q][lane];
         ok = ld_acquire(&A.ctl->done[d]) >= ntask[d];
     }
@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
         int nt = step_ntasks<S, B>(P, A, ph, blockDim.x, workers);
         if (nt == 0 && (A.fixed || !ph.bulk) && ph.ndep > 0) nt = 1;
         ntask[p] = nt;
-        deps.n[p] = ph.ndep;
+        deps.n[p] = ph.ndep | (ph.after + 1) << 8;
         for (int k = 0; k < ph.ndep; k++) deps.d[p][k] = (unsigned short)ph.dep[k];
         cpos[p] = ((A.fixed || !ph.bulk) && nt > 0 && served(ph) == server) ? 1 : 0;
         bfirst[p] = ph.bulk && !A.fixed ? nt : 0;
@@ -494,8 +494,16 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
                 for (int base = h; !got && base < ncp && base < h + 64; base += 32) {
                     const int i = base + lane;
                     const int q = i < ncp ? crit[i] : -1;
-                    const bool avail = q >= 0 && ld_relaxed(&ctl->taken[q]) < ntask[q];
-                    const bool rdy = avail && deps_screen(A, deps, q, ntask);
+                    // an IBM is ready only when every task of its sub-step's sweep
+                    // has been taken too: the phases of a window are looked at one
+                    // after the other, and the dependencies that both share may
+                    // finish in between, so that the sweep is seen waiting and the
+                    // IBM ready
+                    const int sweep = q >= 0 ? (deps.n[q] >> 8) - 1 : -1;
+                    const int taken = q >= 0 ? ld_relaxed(&ctl->taken[q]) : 0;
+                    const int swept = sweep >= 0 ? ld_relaxed(&ctl->taken[sweep]) : 0;
+                    const bool avail = q >= 0 && taken < ntask[q];
+                    const bool rdy = avail && (sweep < 0 || swept >= ntask[sweep]) && deps_screen(A, deps, q, ntask);
                     if (base == h) {  // phases that have nothing left to take leave the window for good
                         const unsigned av = __ballot_sync(FULL, avail);
                         const int nh = av ? base + __ffs(av) - 1 : min(base + 32, ncp);
@@ -591,9 +599,10 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_ste
             return s_go != 0;
         };
         // an IBM task before its stores: the sweep of its sub-step has
-        // finished (no deadlock: that phase is ready whenever the IBM is, and
-        // earlier in the order, so all its tasks were taken before this one,
-        // and a sweep's task never waits after its gate)
+        // finished (no deadlock: all that sweep's tasks were taken before this
+        // one -- the screen asks for it, a task taken before it is ready or by a
+        // fixed owner comes later in the order, and where servers run the IBM the
+        // others take every sweep -- and a sweep's task never waits after its gate)
         auto await = [&]() {
             const int d = A.ph[s_phase].after;
             const bool ok = d < 0 || wait_until(P, A, [&] { return ld_acquire(&A.ctl->done[d]) >= ntask[d]; });

@@ -111,3 +111,22 @@ def test_task_sizes_do_not_change_results(make, threads, rounds, crit):
     for a, b in zip(res[0][0], res[1][0]):
         assert np.array_equal(a, b)
     assert np.array_equal(res[0][1], res[1][1])
+
+
+def test_more_bodies_than_thread_blocks():
+    """no thread block is set apart for a body, and every one may hold an IBM task that awaits a sweep: the sweep's
+    tasks are taken first, so the step completes and equals the graphs"""
+    from paper_2402_04606_gb300.native import TUNE_PERSISTENT, Batch
+
+    spec = wl.cylinder(D=10, levels=2, block=8, storage=wl.F32, n_markers=31, lx=14.0, ly=8.0, xc=4.0)
+    n, res = 500, []  # at most 3 thread blocks on each of 152 SMs
+    for persistent in (1, 0):
+        b = Batch(n, block=8, storage=wl.F32)
+        b.set_tuning(TUNE_PERSISTENT, persistent)
+        members = [b.admit(spec) for _ in range(n)]
+        b.step(40)
+        res.append((members[0].populations(1), [m.forces() for m in members[::71]]))
+        b.close()
+    assert np.array_equal(res[0][0], res[1][0])
+    for x, y in zip(res[0][1], res[1][1]):
+        assert np.array_equal(x, y) and np.array_equal(x, res[0][1][0])

@@ -664,12 +664,11 @@ cudaError_t launch_step_k(const DevPool& P, const StepArgs& A, int grid, int thr
     return cudaLaunchKernelEx(&cfg, kern, P, A);
 }
 
-template <class S, class C, int B, int COLL>
-int occupancy_k(int threads, size_t smem, size_t* static_smem) {
-    auto kern = k_step<S, C, B, COLL, (B >= 16)>;  // the larger of the two in registers and shared memory
+template <class K>
+int occupancy_of(K kern, int threads, size_t smem, size_t* static_smem) {
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return 0;
-    if (static_smem) *static_smem = fa.sharedSizeBytes;
+    if (static_smem && *static_smem < fa.sharedSizeBytes) *static_smem = fa.sharedSizeBytes;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -680,6 +679,17 @@ int occupancy_k(int threads, size_t smem, size_t* static_smem) {
         return 0;
     }
     return nb;
+}
+
+// thread blocks per SM that either variant has room for: one grid serves both, and
+// which one a launch takes (any_vec) may change from step to step
+template <class S, class C, int B, int COLL>
+int occupancy_k(int threads, size_t smem, size_t* static_smem) {
+    if (static_smem) *static_smem = 0;
+    const int plain = occupancy_of(k_step<S, C, B, COLL, false>, threads, smem, static_smem);
+    if (B < 16) return plain;
+    const int vec = occupancy_of(k_step<S, C, B, COLL, (B >= 16)>, threads, smem, static_smem);
+    return plain < vec ? plain : vec;
 }
 
 // the kernel of the context's block size and collision kind, one storage type

@@ -2004,7 +2004,7 @@ sbot_status setup_inst(sbot_ctx* c, int ii, const sbot_domain_desc* desc, const 
     int side = (int)std::ceil(2 * R) + 6;
     int cap = side * side;
     const size_t smem = ibm_smem_bytes(c->storage, cap, hb.n);
-    if (ibm_size_bytes(c->storage, cap, hb.n) > ibm_smem_limit(c->storage))
+    if (ibm_size_bytes(c->storage, cap, hb.n) > ibm_admit_limit() || smem > ibm_smem_limit(c->storage))
         return fail(c, SBOT_ERR_ARG, "body too large for the one-block IBM kernel");
     I.ibm_smem = smem;
     I.has_body = true;

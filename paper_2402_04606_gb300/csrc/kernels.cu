@@ -740,12 +740,27 @@ size_t ibm_size_bytes(int storage, int patch_cap, int n_markers) {
            al16(W * 4) + al16((W + 1) * 4) + al16(ncap * 4) + al16(4 * ncap * c) + 2 * al16(ncap * c);
 }
 
-size_t ibm_smem_limit(int storage) {
-    // the device's opt-in shared memory per block less k_ibm's static shared memory
+// the device's opt-in shared memory per block, 0 when it cannot be asked
+static size_t optin_smem() {
     int dev = 0, optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess || optin <= 0)
-        return 220 * 1024;
+        return 0;
+    return (size_t)optin;
+}
+
+size_t ibm_admit_limit() {
+    // less 1152 bytes of fixed arrays: a line of its own, so that what a body may
+    // be does not move with k_ibm's static shared memory (now 1280; its launches
+    // take less than ibm_size_bytes by more than the difference)
+    const size_t optin = optin_smem();
+    return optin > 0 ? optin - 1152 : 220 * 1024;
+}
+
+size_t ibm_smem_limit(int storage) {
+    // the device's opt-in shared memory per block less k_ibm's static shared memory
+    const size_t optin = optin_smem();
+    if (optin == 0) return 220 * 1024;
     size_t stat = 0;
     dispatch(storage, [&](auto* sp, auto* cp) {
         using S = std::remove_pointer_t<decltype(sp)>;
@@ -753,7 +768,7 @@ size_t ibm_smem_limit(int storage) {
         cudaFuncAttributes fa{};
         stat = cudaFuncGetAttributes(&fa, k_ibm<S, C, 0>) == cudaSuccess ? fa.sharedSizeBytes : 4096;
     });
-    return (size_t)optin > stat ? (size_t)optin - stat : 0;
+    return optin > stat ? optin - stat : 0;
 }
 
 void launch_pose(const DevPool& P, const int* inst_list, const int* pn, int cap, sbot_stream_t s) {

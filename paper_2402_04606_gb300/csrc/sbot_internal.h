@@ -176,6 +176,7 @@ void launch_ibm_geom(int storage, const DevPool& P, const int* inst_list, const 
                      size_t smem, sbot_stream_t s);
 size_t ibm_smem_bytes(int storage, int patch_cap, int n_markers);
 size_t ibm_size_bytes(int storage, int patch_cap, int n_markers);  // at least that: what the admission limit counts
+size_t ibm_admit_limit();            // the largest ibm_size_bytes of a body that is admitted
 size_t ibm_smem_limit(int storage);  // largest dynamic shared memory k_ibm can launch with
 size_t ibm_cache_bytes(int storage, int patch_cap, int n_markers);
 void launch_export(int storage, const DevPool& P, const int* list, int n, const void* f, const void* ffine, int level,

@@ -301,7 +301,8 @@ sbot_status sbot_get_profile(sbot_ctx_t ctx, int kind, int64_t* launches, double
  * tasks started and ended (device time) and how many ran.
  * sbot_get_step_trace returns the last traced step: per phase its kind
  * (0 poses, 1 IBM geometry, 2 coarse-to-fine copy, 3 stream-collide sweep,
- * 4 IBM, 5 force sums), level, queue (1 bulk, 0 critical), tasks, and in
+ * 4 IBM, 5 force sums, 6 collision of the cells a body forces where that is a
+ * phase of its own, in FP64), level, queue (1 bulk, 0 critical), tasks, and in
  * us4[4 p .. 4 p + 3] the first task's start, the last task's start, the
  * first task's end and the last task's end, in microseconds after the
  * launch's first thread block started (-1 for a phase that ran no task),

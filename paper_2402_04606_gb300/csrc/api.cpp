@@ -177,8 +177,7 @@ struct sbot_ctx {
     cudaStream_t gstream[SBOT_MAXLEV] = {};
     cudaEvent_t ev_gfork = nullptr, ev_gjoin[SBOT_MAXLEV] = {};
     cudaStream_t pstream[SBOT_MAXLEV] = {};  // per group: the poses of the coarse step, ahead of its IBM launches
-    cudaEvent_t ev_pose[SBOT_MAXLEV] = {};
-    cudaEvent_t ev_ibm_last[SBOT_MAXLEV] = {}, ev_fsum[SBOT_MAXLEV] = {};  // the step's force sums, off the chain
+    cudaEvent_t ev_ibm[SBOT_MAXLEV] = {}, ev_fsum[SBOT_MAXLEV] = {};  // a sub-step's IBM; the step's force sums
     int ibm_left[SBOT_MAXLEV] = {};  // IBM launches still to record in the coarse step being captured
     int gsub[SBOT_MAXLEV] = {};      // sub-steps of each level recorded so far in the group being captured
     cudaStream_t side[NGL] = {};
@@ -1195,8 +1194,7 @@ sbot_status refresh_groups(sbot_ctx* c) {
         CK(cudaStreamCreateWithPriority(&c->gstream[g], cudaStreamNonBlocking, prio_high));
         CK(cudaEventCreateWithFlags(&c->ev_gjoin[g], cudaEventDisableTiming));
         CK(cudaStreamCreateWithPriority(&c->pstream[g], cudaStreamNonBlocking, prio_high));
-        CK(cudaEventCreateWithFlags(&c->ev_pose[g], cudaEventDisableTiming));
-        CK(cudaEventCreateWithFlags(&c->ev_ibm_last[g], cudaEventDisableTiming));
+        CK(cudaEventCreateWithFlags(&c->ev_ibm[g], cudaEventDisableTiming));
         CK(cudaEventCreateWithFlags(&c->ev_fsum[g], cudaEventDisableTiming));
         for (int l = 0; l <= g; l++) {
             const int gl = gl_of(g + 1, l);
@@ -1280,10 +1278,17 @@ void drop_graph(sbot_ctx* c, int g) {
 
 // One substep of level l of every instance of group g (m = g + 1 levels) and,
 // recursively, two of every finer level: Algorithm 1 with each stream+collide
-// pair fused into one pull kernel, on the group's stream; then the IBM of the
-// level's bodies.  Blocks that need no finer level and that no body touches run on a
-// side stream from the start of the substep, beside both.  Launch sizes are the list
-// capacities; the kernels read the current lengths on the device.
+// pair fused into one pull kernel, on the group's stream.  Blocks that need no
+// finer level and that no body touches run on a side stream from the start of the
+// substep; so does the IBM of the level's bodies on the pose stream, and when it and
+// the sweep of the other blocks are over, the stencil cells are collided again with
+// their force.  Launch sizes are the list capacities; the kernels read the current
+// lengths on the device.
+// (us per coarse step with the IBM, and its own collision of the cells, after both
+// sweeps -> after the sweep of the blocks they touch -> now: immersed cylinder in a
+// cavity 46.1 -> 38.9 -> 31.8; D = 40 cylinder 104.5 -> 93.4 -> 84.2, in FP64 411
+// -> 252; D = 128 433 -> 413 -> 339; flapping ellipse 263 -> 242 -> 217; 64
+// instances in BF16 1115 -> 1067 -> 1027)
 void advance(sbot_ctx* c, const DevPool& P, int g, int l) {
     const int storage = c->storage, gl = gl_of(g + 1, l);
     // a profiled step is captured on the context stream alone, so that the
@@ -1303,11 +1308,26 @@ void advance(sbot_ctx* c, const DevPool& P, int g, int l) {
     // finer region own the copied values, writes the halo (fold)
     const int sub = c->gsub[l]++;
     void* fold = (l < g && sub + 1 < (1 << l)) ? fine : nullptr;
+    const WorkList& Wb = W_of(c, gl, LK_IBM);
+    auto ibm = [&](cudaStream_t s) {
+        launch_ibm(storage, P, lptr(c, gl, LK_IBM), cptr(c, gl, LK_IBM), Wb.cap, cur, l, 0, c->ibm_smem[g], s, 1,
+                   c->ibm_threads);
+    };
+    auto force_sum = [&](cudaStream_t s) {  // after the coarse step's last IBM: beside the rest
+        if (--c->ibm_left[g] == 0)
+            launch_force_sum(storage, P, lptr(c, gl, LK_IBM), cptr(c, gl, LK_IBM), Wb.cap, 1 << g, s);
+    };
+    if (!serial && (fork || Wb.cap > 0)) cudaEventRecord(c->ev_fork[gl], st);
+    if (!serial && Wb.cap > 0) {  // the pose stream: behind a moving body's geometry, and the last step's force sums
+        cudaStream_t sp = c->pstream[g];
+        cudaStreamWaitEvent(sp, c->ev_fork[gl], 0);
+        ibm(sp);
+        cudaEventRecord(c->ev_ibm[g], sp);
+        force_sum(sp);
+        cudaEventRecord(c->ev_fsum[g], sp);
+    }
     if (fork) {
-        if (!serial) {
-            cudaEventRecord(c->ev_fork[gl], st);
-            cudaStreamWaitEvent(sd, c->ev_fork[gl], 0);
-        }
+        if (!serial) cudaStreamWaitEvent(sd, c->ev_fork[gl], 0);
         {
             ProfScope ps(c, 0, gl, LK_INDEP, sd);
             launch_fused(storage, P, lptr(c, gl, LK_INDEP), cptr(c, gl, LK_INDEP), Wi.cap, Wi.cap, c->vec_min_cells, c->staged, cur,
@@ -1340,29 +1360,13 @@ void advance(sbot_ctx* c, const DevPool& P, int g, int l) {
         launch_fused(storage, P, lptr(c, gl, LK_FUSED), cptr(c, gl, LK_FUSED), Wf.cap, Wf.cap,
                      l < g ? -1 : c->vec_min_cells, c->staged, cur, nxt, fine, l, st, fold);
     }
-    // the bodies on this level: after the sweep of the blocks they force, whose
-    // unforced cells the IBM collides again with their force.  The side stream's
-    // blocks are none of theirs and go on beside it: they are waited for only after
-    // it (waited for before it, us per coarse step in the graphs: immersed cylinder
-    // in a cavity 46.2, now 38.9; D = 40 cylinder 103.5 -> 93.4; flapping ellipse
-    // 264 -> 242; 64 instances in BF16 with the vector sweep from 65536 cells on
-    // 1318 -> 1218)
-    const WorkList& Wb = W_of(c, gl, LK_IBM);
-    if (Wb.cap > 0) {
-        if ((c->moving >> g) & 1) cudaStreamWaitEvent(st, c->ev_pose[g], 0);
-        {
-            ProfScope ps(c, 3, gl, LK_IBM, st);
-            launch_ibm(storage, P, lptr(c, gl, LK_IBM), cptr(c, gl, LK_IBM), Wb.cap, cur, nxt, l, 0, c->ibm_smem[g], st, 1,
-                       c->ibm_threads);
-        }
-        if (--c->ibm_left[g] == 0) {  // the coarse step's last IBM: its force sums run beside the rest
-            cudaStream_t sp = serial ? st : c->pstream[g];
-            cudaEventRecord(c->ev_ibm_last[g], st);
-            cudaStreamWaitEvent(sp, c->ev_ibm_last[g], 0);
-            launch_force_sum(storage, P, lptr(c, gl, LK_IBM), cptr(c, gl, LK_IBM), Wb.cap, 1 << g, sp);
-            cudaEventRecord(c->ev_fsum[g], sp);
-        }
+    if (Wb.cap > 0) {  // the side stream's blocks are none of the bodies' and go on beside this
+        if (!serial) cudaStreamWaitEvent(st, c->ev_ibm[g], 0);
+        ProfScope ps(c, 3, gl, LK_IBM, st);
+        if (serial) ibm(st);
+        launch_forced(storage, P, lptr(c, gl, LK_IBM), cptr(c, gl, LK_IBM), Wb.cap, cur, nxt, l, st);
     }
+    if (Wb.cap > 0 && serial) force_sum(st);
     if (fork && !serial) cudaStreamWaitEvent(st, c->ev_join[gl], 0);
     c->par[l] ^= 1;
 }
@@ -1387,7 +1391,6 @@ void advance_all(sbot_ctx* c) {
             // the IBM geometry of every finest step of this coarse step, ahead of the IBM launches
             launch_ibm_geom(c->storage, P, lptr(c, glb, LK_IBM), cptr(c, glb, LK_IBM), W_of(c, glb, LK_IBM).cap,
                             1 << g, c->ibm_smem[g], ps);
-            cudaEventRecord(c->ev_pose[g], ps);
         }
         const bool bodies = W_of(c, glb, LK_IBM).cap > 0;
         c->ibm_left[g] = bodies ? 1 << g : -1;
@@ -1406,6 +1409,10 @@ void advance_all(sbot_ctx* c) {
 // the persistent step: Algorithm 1 as a phase list for the step kernel
 // ---------------------------------------------------------------------------
 
+// tasks per body of a forced collision that is a phase of its own: an SM collides 64
+// cells in FP64 in about 3 us, and a body has 300 to 1900
+constexpr int FORCED_TASKS = 16;
+
 // The phases of one coarse step of group g (its instances have m = g + 1
 // levels), in the order of Algorithm 1 as advance() launches them, each with
 // the phases it must wait for:
@@ -1415,18 +1422,21 @@ void advance_all(sbot_ctx* c) {
 //   sweep of level l, blocks needing no finer level and away from a body's
 //     stencils (A): the level's previous sweep (neighbours; the buffer it
 //     overwrites) and the copy into level l (halo cells);
-//   the other blocks (B): the same, plus the level's previous IBM (the cells it
-//     collided) and the two sweeps of level l+1 (whose halo values the coarse
-//     pull merges);
+//   the other blocks (B): the same, plus the level's previous forced collision
+//     (of the stencil cells, by the IBM itself or after it) and the two sweeps of
+//     level l+1 (whose halo values the coarse pull merges);
 //   IBM of a finest sub-step: whatever B waits for (the pre-collision state it
-//     pulls) and, for a moving body, the geometry of that step; its stores wait
-//     for B, whose unforced values they replace.
+//     pulls) and, for a moving body, the geometry of that step; its stores of the
+//     cells wait for B, whose unforced values they replace;
+//   forced collision, where it is a phase of its own (FP64, STEP_LIST_BYTES):
+//     the IBM and B.
 struct PhaseEmit {
     sbot_ctx* c;
     int g;
     std::vector<StepPhase> ph;
     int lastA[SBOT_MAXLEV], lastB[SBOT_MAXLEV], c2f_into[SBOT_MAXLEV], par[SBOT_MAXLEV], sub[SBOT_MAXLEV];
     int last_ibm = -1, n_ibm = 0;
+    int last_forced = -1;    // the phase that collided the stencil cells last: the IBM, or the one after it
     int prev_fsum = -1;  // the previous coarse step's force sums (their term slots are the next IBMs')
     bool bodies = false, moving = false;
     std::vector<int> geom;
@@ -1473,7 +1483,7 @@ struct PhaseEmit {
         }
         const int c2 = l > 0 ? c2f_into[l] : -1;
         const int fa = l < g ? lastA[l + 1] : -1, fb = l < g ? lastB[l + 1] : -1;
-        const int forced = l == g ? last_ibm : -1;  // the level's previous IBM wrote the cells this sweep pulls
+        const int forced = l == g ? last_forced : -1;  // it wrote the cells this sweep pulls
         int A = -1, Bp;
         if (fork) {
             // (static bodies: the list's blocks neither pull nor overwrite a cell that the IBM touches, build_topology)
@@ -1488,12 +1498,16 @@ struct PhaseEmit {
             // it may start when the sweep may (it waits for whatever the
             // sweep waits for), and waits for the sweep before its stores
             ph[Bp].bulk = -1;
-            const int ibm = add(PH_IBM, l, gl, LK_IBM,
-                                {lastA[l], lastB[l], c2, last_ibm, moving ? geom[n_ibm] : -1,
-                                 n_ibm == 0 ? prev_fsum : -1}, cur, nxt, -1, n_ibm);
-            ph[ibm].after = Bp;
+            last_ibm = add(PH_IBM, l, gl, LK_IBM,
+                           {lastA[l], lastB[l], c2, forced, moving ? geom[n_ibm] : -1, n_ibm == 0 ? prev_fsum : -1},
+                           cur, nxt, -1, n_ibm);
             n_ibm++;
-            last_ibm = ibm;
+            if (storage_bytes(c->storage) == STEP_LIST_BYTES) {
+                last_forced = add(PH_FORCED, l, gl, LK_IBM, {last_ibm, Bp}, cur, nxt, -1, FORCED_TASKS);
+            } else {
+                ph[last_ibm].after = Bp;
+                last_forced = last_ibm;
+            }
         }
         if (fold && Bp >= 0) {
             ph[Bp].fold = 1;
@@ -1520,7 +1534,7 @@ struct PhaseEmit {
             n_ibm = 0;
             geom.clear();
             if (moving) {
-                const int pose = add(PH_POSE, g, glb, LK_IBM, {last_ibm});
+                const int pose = add(PH_POSE, g, glb, LK_IBM, {last_forced});
                 for (int i = 0; i < (1 << g); i++)
                     geom.push_back(add(PH_GEOM, g, glb, LK_IBM, {pose}, -1, -1, -1, i));
             }
@@ -1774,7 +1788,7 @@ sbot_status finalize_inst(sbot_ctx* c, int ii) {
     if (I.has_body) {
         const int one[2] = {ii, 1};  // an instance list of one entry, and its length
         TRY(upload(c, c->d_one, one, sizeof one));
-        launch_ibm(c->storage, P, c->d_one, c->d_one + 1, 1, pre_buf(c, fin), nullptr, fin, 1, I.ibm_smem, c->s);
+        launch_ibm(c->storage, P, c->d_one, c->d_one + 1, 1, pre_buf(c, fin), fin, 1, I.ibm_smem, c->s);
         c->launch_n++;
         CK(cudaGetLastError());
     }
@@ -2829,8 +2843,7 @@ sbot_status sbot_destroy(sbot_ctx_t c) {
         if (c->ev_gjoin[g]) cudaEventDestroy(c->ev_gjoin[g]);
         if (c->pstream[g]) cudaStreamSynchronize(c->pstream[g]);
         if (c->pstream[g]) cudaStreamDestroy(c->pstream[g]);
-        if (c->ev_pose[g]) cudaEventDestroy(c->ev_pose[g]);
-        if (c->ev_ibm_last[g]) cudaEventDestroy(c->ev_ibm_last[g]);
+        if (c->ev_ibm[g]) cudaEventDestroy(c->ev_ibm[g]);
         if (c->ev_fsum[g]) cudaEventDestroy(c->ev_fsum[g]);
     }
     if (c->ev_gfork) cudaEventDestroy(c->ev_gfork);

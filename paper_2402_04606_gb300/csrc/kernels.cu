@@ -370,10 +370,10 @@ __global__ void __launch_bounds__(IBM_THREADS) k_ibm_geom(const __grid_constant_
     ibm_geom_run<C>(P, ilist[item], blockIdx.y, smraw, sh);
 }
 
-template <class S, class C, int COLL>
+template <class S, class C>
 __global__ void __launch_bounds__(IBM_THREADS) k_ibm(const __grid_constant__ DevPool P, const int* __restrict__ ilist,
                                                      const int* __restrict__ pn, const S* __restrict__ fin,
-                                                     S* __restrict__ fout, int level, int direct, int deferred) {
+                                                     int level, int direct, int deferred) {
     pdl_enter();
     const int item = blockIdx.x;
     if (item >= *pn) return;
@@ -381,9 +381,21 @@ __global__ void __launch_bounds__(IBM_THREADS) k_ibm(const __grid_constant__ Dev
     __shared__ IbmShared sh;
     if (threadIdx.x == 0) sh.geo_inst = -1;
     __syncthreads();
-    // launched after the sub-step's sweep on the same stream
-    ibm_run<S, C, COLL>(P, ilist[item], fin, fout, level, direct, deferred, -1, smraw, sh, [] { return true; },
-                        [] {}, [] { return true; });
+    ibm_run<S, C, 0, true, sizeof(C) == 4>(P, ilist[item], fin, nullptr, level, direct, deferred, -1, smraw, sh,
+                                           [] { return true; }, [] {}, [] { return true; });
+}
+
+// 64 threads a block and 32 blocks a body: 2000 cells (a body of 400 markers) in
+// one pass, on as many SMs as there are blocks, which FP64 needs
+#define FORCED_THREADS 64
+#define FORCED_PARTS 32
+template <class S, class C, int COLL>
+__global__ void __launch_bounds__(FORCED_THREADS) k_forced(const __grid_constant__ DevPool P,
+                                                           const int* __restrict__ ilist, const int* __restrict__ pn,
+                                                           const S* __restrict__ fin, S* __restrict__ fout, int level) {
+    pdl_enter();
+    if ((int)blockIdx.y >= *pn) return;
+    ibm_forced_run<S, C, COLL>(P, ilist[blockIdx.y], fin, fout, level, blockIdx.x, gridDim.x);
 }
 
 template <class C>
@@ -766,7 +778,7 @@ size_t ibm_smem_limit(int storage) {
         using S = std::remove_pointer_t<decltype(sp)>;
         using C = std::remove_pointer_t<decltype(cp)>;
         cudaFuncAttributes fa{};
-        stat = cudaFuncGetAttributes(&fa, k_ibm<S, C, 0>) == cudaSuccess ? fa.sharedSizeBytes : 4096;
+        stat = cudaFuncGetAttributes(&fa, k_ibm<S, C>) == cudaSuccess ? fa.sharedSizeBytes : 4096;
     });
     return optin > stat ? optin - stat : 0;
 }
@@ -800,28 +812,33 @@ void launch_force_sum(int storage, const DevPool& P, const int* inst_list, const
     });
 }
 
-template <class S, class C, int COLL>
-void launch_ibm_k(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, const void* f, void* fout,
-                  int level, int direct, size_t smem, sbot_stream_t s, int deferred, int threads) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaFuncSetAttribute(k_ibm<S, C, COLL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)ibm_smem_limit(storage));
-        attr_set = true;
-    }
-    launch_k(P.pdl, k_ibm<S, C, COLL>, dim3(cap), dim3(threads > 0 && threads <= IBM_THREADS ? threads : IBM_THREADS),
-             smem, s, P, inst_list, pn, (const S*)f, (S*)fout, level, direct, deferred);
-}
-
-void launch_ibm(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, const void* f, void* fout,
+void launch_ibm(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, const void* f,
                 int level, int direct, size_t smem, sbot_stream_t s, int deferred, int threads) {
     if (cap <= 0) return;
     dispatch(storage, [&](auto* sp, auto* cp) {
         using S = std::remove_pointer_t<decltype(sp)>;
         using C = std::remove_pointer_t<decltype(cp)>;
+        static bool attr_set = false;
+        if (!attr_set) {
+            cudaFuncSetAttribute(k_ibm<S, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)ibm_smem_limit(storage));
+            attr_set = true;
+        }
+        launch_k(P.pdl, k_ibm<S, C>, dim3(cap), dim3(threads > 0 && threads <= IBM_THREADS ? threads : IBM_THREADS),
+                 smem, s, P, inst_list, pn, (const S*)f, level, direct, deferred);
+    });
+}
+
+void launch_forced(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, const void* fin,
+                   void* fout, int level, sbot_stream_t s) {
+    if (cap <= 0) return;
+    dispatch(storage, [&](auto* sp, auto* cp) {
+        using S = std::remove_pointer_t<decltype(sp)>;
+        using C = std::remove_pointer_t<decltype(cp)>;
         const int k = P.coll & 15;
-        (k == 1 ? launch_ibm_k<S, C, 1> : (k == 2 ? launch_ibm_k<S, C, 2> : launch_ibm_k<S, C, 0>))(
-            storage, P, inst_list, pn, cap, f, fout, level, direct, smem, s, deferred, threads);
+        auto kern = k == 1 ? k_forced<S, C, 1> : (k == 2 ? k_forced<S, C, 2> : k_forced<S, C, 0>);
+        launch_k(P.pdl, kern, dim3(FORCED_PARTS, cap), dim3(FORCED_THREADS), 0, s, P, inst_list, pn, (const S*)fin,
+                 (S*)fout, level);
     });
 }
 

@@ -1799,28 +1799,84 @@ __device__ __noinline__ C ibm_pull(const DevPool& P, const S* fin, int slot, con
                                    int y, int q) {
     return pull_int<S, C>(P, fin, nullptr, false, slot, ip, level, x, y, q);
 }
+// where a marker box lies and its slot table (IbmCacheHead)
+struct IbmBox {
+    bool table;
+    int px0, py0, pnbx, pbx0, pby0;
+    const int* pslot;
+};
+__device__ __forceinline__ IbmBox ibm_box(const IbmCacheHead& hd, const int* pslot) {
+    return IbmBox{hd.table != 0, hd.px0, hd.py0, hd.pnbx, hd.pbx0, hd.pby0, pslot};
+}
+// The pre-collision populations of stencil cell c (x | y << 16 in the box) in
+// compute form, and the index of its population 0 (-1: not a finest interior cell
+// with a source in every direction).  direct: the populations as they are, not
+// pulled.  par: what holds the shift of 16-bit storage.
+template <class S, class C, class Par>
+__device__ __forceinline__ long long ibm_cell(const DevPool& P, const InstParams& ip, const Par& par, int level,
+                                              const IbmBox& bx, const S* fin, int c, bool direct, C* v) {
+    const int B = P.B, BB = B * B, lb = 31 - __clz(B);
+    const int gx = bx.px0 + (c & 0xffff), gy = bx.py0 + (c >> 16);
+    if (bx.table) {
+        const int* const ps = bx.pslot + 9 * (((gy >> lb) - bx.pby0) * bx.pnbx + (gx >> lb) - bx.pbx0);
+        const int x = gx & (B - 1), y = gy & (B - 1), slot = ps[4];
+        if (slot < 0) return -1;
+        const long long own = (long long)slot * 9 * BB + y * B + x;
+        bool ok = true;
+#pragma unroll
+        for (int q = 0; q < 9; q++) {
+            if (direct) {
+                v[q] = Sto<S>::template ld<C>(fin, own + q * BB, q, par.dref);
+                continue;
+            }
+            const int sx = x - CXq(q), sy = y - CYq(q);
+            const int dx = sx < 0 ? -1 : (sx >= B ? 1 : 0), dy = sy < 0 ? -1 : (sy >= B ? 1 : 0);
+            const int ns = ps[(dy + 1) * 3 + dx + 1];
+            ok &= ns >= 0;
+            v[q] = Sto<S>::template ld<C>(
+                fin, ((size_t)max(ns, 0) * 9 + q) * BB + (sy & (B - 1)) * B + (sx & (B - 1)), q, par.dref);
+        }
+        return ok ? own : -1;
+    }
+    const int slot = lat_slot(P, ip, level, gx, gy);
+    if (slot < 0 || P.slot_type[slot] != ST_INT) return -1;
+    const int x = gx - P.slot_ox[slot], y = gy - P.slot_oy[slot];
+    const long long own = (long long)slot * 9 * BB + y * B + x;
+#pragma unroll
+    for (int q = 0; q < 9; q++)
+        v[q] = direct ? Sto<S>::template ld<C>(fin, own + q * BB, q, ip.dref)
+                      : ibm_pull<S, C>(P, fin, slot, ip, level, x, y, q);
+    return own;
+}
 // One body's IBM step (k_ibm runs one per thread block); smraw is the
 // block's dynamic shared memory (ibm_smem_bytes), sh its fixed part.
 // direct (the state at t = 0): reads the pre-collision state as it is and
 // leaves the force field in the instance's patch for the first collision.
-// Else it pulls the stencil cells' pre-collision populations from fin, and
-// once it has their force it collides them (Eqs. 3, 6-8) and stores them in
-// fout, over the unforced values this sub-step's sweep wrote there: the sweep
-// then never waits for the IBM, nor the IBM for the sweep until its last
-// stores.  (With the forced blocks swept after the IBM, every finest step was
-// a chain IBM - hand-over - sweep - hand-over.  With the servers of
-// step_impl.cuh, us per coarse step: D = 40 cylinder 63.6 -> 48.7, flapping
-// ellipse 182 -> 148, pitching section 103 -> 82, immersed cylinder in a cavity,
-// 382 markers, 38.7 -> 33.)
+// Else it pulls the stencil cells' pre-collision populations from fin; the
+// cells are collided with their force (Eqs. 3, 6-8) and stored in fout, over the
+// unforced values this sub-step's sweep wrote there, so that the sweep never
+// waits for the IBM, nor the IBM for the sweep.  (With the forced blocks swept
+// after the IBM, every finest step was a chain IBM - hand-over - sweep -
+// hand-over.  With the servers of step_impl.cuh, us per coarse step: D = 40
+// cylinder 63.6 -> 48.7, flapping ellipse 182 -> 148, pitching section 103 ->
+// 82, immersed cylinder in a cavity, 382 markers, 38.7 -> 33.)
+// LIST: the forces are left in the patch, one pair per stencil cell, and
+// ibm_forced_run collides the cells, on many SMs, once the sweep is over too: in
+// the graphs, where a launch is the only way to wait for the sweep, and in FP64,
+// of which an SM does two operations a cycle -- collided by the body's own thread
+// block, 1000 cells took 38 us.  Else the body's thread block collides them:
+// await() is called by one whole warp and waits until the sub-step's sweep has
+// finished; swept(), after a barrier that follows it and before the stores to
+// fout, says whether it has; false: stop.
+// REG: each thread keeps its first cell in registers (k_ibm in FP64, whose 1024
+// threads have 64 each, spilled 724 bytes with it and keeps none).
 // sub: which finest step of the coarse step this is (-1: not known; the
 // geometry is then looked up by the body's step counter).
 // gate(): called once by the whole block, after the part that may run before
 // the step's earlier phases have finished (the load of a stored geometry)
 // and before the first read of their results; false: stop (the launch is
-// aborting).  await(): called by one whole warp: waits until this sub-step's
-// sweep has finished; swept(), after a barrier that follows it and before the
-// stores to fout: whether it has; false: stop.
-template <class S, class C, int COLL, class G, class G1, class G2>
+// aborting).
+template <class S, class C, int COLL, bool LIST, bool REG, class G, class G1, class G2>
 __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int level, int direct, int deferred, int sub,
                         unsigned char* smraw, IbmShared& sh, G&& gate, G1&& await, G2&& swept) {
     const InstParams& ip = P.inst[inst];
@@ -1831,7 +1887,6 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
     const int ncap = ibm_ncap(cap, N), W = (cap + 31) / 32 + 1;
 
     const IbmSmem<C> m = ibm_carve<C>(smraw, N, ncap, W);
-    int* const pslot = m.pslot;
     IbmV2<C>* const F = m.F;
     int* const bb = sh.bb;
     double* const pose = sh.pose;
@@ -1924,12 +1979,14 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
             }
         }
         __syncthreads();
-        if (!ibm_geometry<C>(P, ip, level, pose, still, m, head, bb, wtot)) return;
+        if (!ibm_geometry<C>(P, ip, level, pose, still, m, head, bb, wtot)) {
+            if (LIST && tid == 0) st->forced = -1;
+            return;
+        }
     }
     for (int j = tid; j < N; j += nt) F[j] = IbmV2<C>{(C)0, (C)0};
     __syncthreads();
     const int px0 = head.px0, py0 = head.py0, w = head.w, h = head.h, ncell = head.ncell;
-    const bool table = head.table != 0;
     const int* const ccell = m.ccell;
     const int* const cst = m.cst;
     const IbmEnt<C>* const ent = m.ent;
@@ -1941,43 +1998,9 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
     IbmV2<C>* const cu = m.cu;
     IbmV2<C>* const cF = m.cF;
     C* const cinv = m.cinv;
-    const int lb = 31 - __clz(B), BB = B * B, pnbx = head.pnbx, pbx0 = head.pbx0, pby0 = head.pby0;
-    // the pre-collision populations of stencil cell ci (compute form) and the
-    // index of its population 0 (-1: not a finest interior cell with a source
-    // in every direction)
-    auto pull = [&](int ci, C* v) -> long long {
-        const int c = ccell[ci], gx = px0 + (c & 0xffff), gy = py0 + (c >> 16);
-        if (table) {
-            const int* const ps = pslot + 9 * (((gy >> lb) - pby0) * pnbx + (gx >> lb) - pbx0);
-            const int x = gx & (B - 1), y = gy & (B - 1), slot = ps[4];
-            if (slot < 0) return -1;
-            const long long own = (long long)slot * 9 * BB + y * B + x;
-            bool ok = true;
-#pragma unroll
-            for (int q = 0; q < 9; q++) {
-                if (direct) {
-                    v[q] = Sto<S>::template ld<C>(fin, own + q * BB, q, par.dref);
-                    continue;
-                }
-                const int sx = x - CXq(q), sy = y - CYq(q);
-                const int dx = sx < 0 ? -1 : (sx >= B ? 1 : 0), dy = sy < 0 ? -1 : (sy >= B ? 1 : 0);
-                const int ns = ps[(dy + 1) * 3 + dx + 1];
-                ok &= ns >= 0;
-                v[q] = Sto<S>::template ld<C>(
-                    fin, ((size_t)max(ns, 0) * 9 + q) * BB + (sy & (B - 1)) * B + (sx & (B - 1)), q, par.dref);
-            }
-            return ok ? own : -1;
-        }
-        const int slot = lat_slot(P, ip, level, gx, gy);
-        if (slot < 0 || P.slot_type[slot] != ST_INT) return -1;
-        const int x = gx - P.slot_ox[slot], y = gy - P.slot_oy[slot];
-        const long long own = (long long)slot * 9 * BB + y * B + x;
-#pragma unroll
-        for (int q = 0; q < 9; q++)
-            v[q] = direct ? Sto<S>::template ld<C>(fin, own + q * BB, q, ip.dref)
-                          : ibm_pull<S, C>(P, fin, slot, ip, level, x, y, q);
-        return own;
-    };
+    const int BB = B * B;
+    const IbmBox box = ibm_box(head, m.pslot);
+    auto pull = [&](int ci, C* v) { return ibm_cell<S, C>(P, ip, par, level, box, fin, ccell[ci], direct != 0, v); };
     // uncorrected moments of the pre-collision state on the stencil cells (Sec. 2.2 after Eq. 11)
     auto moments = [&](int ci, C* v, IbmV2<C>& u, C& inv) -> long long {
         C r = 1, jx = 0, jy = 0;
@@ -2011,7 +2034,7 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
     for (int i = 0; i < IBM_RE; i++) ew[i] = 0;
 #pragma unroll
     for (int i = 0; i < IBM_RE / 2; i++) em[i] = 0;
-    if (tid < ncell) {
+    if (REG && tid < ncell) {
         own0 = moments(tid, f0, u0, inv0);
         e0 = cst[tid];
         e1 = cst[tid + 1];
@@ -2024,7 +2047,8 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
             }
         }
     }
-    for (int ci = tid + nt; ci < ncell; ci += nt) {
+    const int rest = REG ? tid + nt : tid;  // the thread's first cell that is not in registers
+    for (int ci = rest; ci < ncell; ci += nt) {
         C v[9], inv;
         IbmV2<C> u;
         moments(ci, v, u, inv);
@@ -2063,7 +2087,7 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
             F[j] = fj;
         }
         __syncthreads();
-        if (tid < ncell) {
+        if (REG && tid < ncell) {
             C sx = 0, sy = 0;
 #pragma unroll
             for (int h = 0; h < IBM_RE; h += 4) {
@@ -2092,7 +2116,7 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
             u0.y += sy * inv0;
             cu[tid] = u0;
         }
-        for (int ci = tid + nt; ci < ncell; ci += nt) {
+        for (int ci = rest; ci < ncell; ci += nt) {
             C sx = 0, sy = 0;
             const int b1 = cst[ci + 1];
             for (int e = cst[ci]; e < b1; e++) {
@@ -2124,14 +2148,19 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
         __syncthreads();
         for (int ci = tid; ci < ncell; ci += nt) {
             const int c = (ccell[ci] >> 16) * w + (ccell[ci] & 0xffff);
-            const IbmV2<C> g = ci == tid ? F0 : cF[ci];
+            const IbmV2<C> g = REG && ci == tid ? F0 : cF[ci];
             gF[c] = g.x;
             gF[cap + c] = g.y;
         }
+    } else if (LIST) {
+        IbmV2<C>* const gF = (IbmV2<C>*)ip.patch;
+        for (int ci = tid; ci < ncell; ci += nt) gF[ci] = REG && ci == tid ? F0 : cF[ci];
     }
-    // a static body keeps its geometry for the next launches
-    if (still && ip.ibm_cache != nullptr && stored == nullptr)
-        ibm_store((IbmCacheHead*)ip.ibm_cache, head, smraw, m.cache_bytes, -1);
+    // a static body keeps its geometry for the next launches; for the cells' list
+    // that follows, a moving one whose geometry was not stored (which the steps'
+    // order rules out) leaves it in its first entry
+    if (stored == nullptr && ip.ibm_cache != nullptr && (still || (LIST && !direct)))
+        ibm_store((IbmCacheHead*)ip.ibm_cache, head, smraw, m.cache_bytes, !LIST || still ? -1 : k);
     // Eq. 16 and the moment about the pivot: per-marker terms in the compute
     // type; inside the step graph they are stored and summed for the whole
     // coarse step by k_force_sum, off the critical path (FP64 runs at a small
@@ -2157,7 +2186,7 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
     } else {
         ibm_force_sum<C>(N, terms, red, ip.hist + 3 * (k % SBOT_HIST_CAP));
     }
-    if (!direct) {
+    if (!LIST && !direct) {
         // the forced collision of the stencil cells (an inlet cell keeps the
         // sweep's value: it is reset to the inlet state after streaming)
         const C om = (C)par.om;
@@ -2186,6 +2215,7 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
     }
     if (tid == 0) {
         sh.geo_inst = still && stored != nullptr ? inst : -1;
+        if (LIST) st->forced = ip.ibm_cache == nullptr ? -1 : !still && stored != nullptr ? (int)(k - st->pose_k0) : 0;
         st->patch_x0 = px0;
         st->patch_y0 = py0;
         st->patch_w = w;
@@ -2195,6 +2225,54 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
             __threadfence();
             st->ibm_cached = 1;
         }
+    }
+}
+// the collision of one cell's populations f with the force (gx, gy).  LES in FP64: a
+// function of its own, so that the graphs' kernel and the step kernel round alike
+// (inlined, it contracted to different fmas in the two; the other collisions do
+// not, and called they cost a D = 40 cylinder's step 4 %)
+template <class S, class C, int COLL>
+__device__ __noinline__ void forced_apart(C* f, C om, C gx, C gy, const InstParams& ip) {
+    collide_k<COLL, C, true, DevTrait<S>::value, sizeof(S) == 4>(f, om, gx, gy, ip);
+}
+template <class S, class C, int COLL>
+__device__ __forceinline__ void forced_collision(C* f, C om, C gx, C gy, const InstParams& ip) {
+    if constexpr (sizeof(S) == STEP_LIST_BYTES && COLL == 2)
+        forced_apart<S, C, COLL>(f, om, gx, gy, ip);
+    else
+        collide_k<COLL, C, true, DevTrait<S>::value, sizeof(S) == 4>(f, om, gx, gy, ip);
+}
+// The forced collision of a body's stencil cells (LIST of ibm_run), part
+// `part` of `parts` of them by this thread block: pulled from fin again, with the
+// forces the patch holds, and stored in fout over what the sweep wrote there (an
+// inlet cell keeps the sweep's value: it is reset to the inlet state after
+// streaming).
+template <class S, class C, int COLL>
+__device__ void ibm_forced_run(const DevPool& P, int inst, const S* fin, S* fout, int level, int part, int parts) {
+    const InstParams& ip = P.inst[inst];
+    const int entry = P.ist[inst].forced;
+    if (entry < 0) return;
+    const IbmCacheHead& hd =
+        *(const IbmCacheHead*)((const unsigned char*)ip.ibm_cache + (size_t)entry * ip.ibm_cache_stride);
+    const int N = ip.n_markers, cap = ip.patch_cap, BB = P.B * P.B, nxl = ip.nx0 << level, nyl = ip.ny0 << level;
+    const IbmSmem<C> m = ibm_carve<C>((unsigned char*)(&hd + 1), N, ibm_ncap(cap, N), (cap + 31) / 32 + 1);
+    const IbmV2<C>* const F = (const IbmV2<C>*)ip.patch;
+    const C om = (C)1 / (C)ip.tau[level];
+    const IbmBox box = ibm_box(hd, m.pslot);
+    // an even share for each part, in whole warps
+    const int ncell = hd.ncell, share = ((ncell + parts - 1) / parts + 31) & ~31;
+    const int end = min(ncell, (part + 1) * share);
+    for (int ci = part * share + threadIdx.x; ci < end; ci += blockDim.x) {
+        const int c = m.ccell[ci], gx = box.px0 + (c & 0xffff), gy = box.py0 + (c >> 16);
+        C f[9];
+        const long long own = ibm_cell<S, C>(P, ip, ip, level, box, fin, c, false, f);
+        if (own < 0 || (gx == 0 && ip.bc[SIDE_W] == BCK_INLET) || (gx == nxl - 1 && ip.bc[SIDE_E] == BCK_INLET) ||
+            (gy == 0 && ip.bc[SIDE_S] == BCK_INLET) || (gy == nyl - 1 && ip.bc[SIDE_N] == BCK_INLET))
+            continue;
+        const IbmV2<C> g = F[ci];
+        forced_collision<S, C, COLL>(f, om, g.x, g.y, ip);
+#pragma unroll
+        for (int q = 0; q < 9; q++) Sto<S>::template st<C>(fout, own + q * BB, q, f[q], ip.dref);
     }
 }
 // The force and moment of Eq. 16 for every finest step of the coarse step

@@ -94,7 +94,7 @@ struct InstState {
     int patch_x0, patch_y0, patch_w, patch_h;
     long long pose_k0;    // finest time of pose_tab[0], -1 before the first table
     int ibm_cached;       // the IBM cache holds this body's geometry
-    int pad;
+    int forced;           // the cache entry of the cells whose forces the patch holds, -1 none (ibm_forced_run)
 };
 
 // Everything a kernel needs, passed by value.
@@ -166,10 +166,12 @@ void launch_pose(const DevPool& P, const int* inst_list, const int* pn, int cap,
 // for launch_force_sum, which sums the `steps` finest steps of the coarse
 // step just run
 // threads: the thread block that runs one body (at most 1024)
-// direct = 0: collides the cells it forces and stores them in fout, over what
-// the sub-step's sweep (launched before it on the same stream) wrote there
+// direct = 0: leaves the forces of its stencil cells for launch_forced, which
+// collides the cells with them, over what the sub-step's sweep wrote in fout
 void launch_ibm(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, const void* f,
-                void* fout, int level, int direct, size_t smem, sbot_stream_t s, int deferred = 0, int threads = 1024);
+                int level, int direct, size_t smem, sbot_stream_t s, int deferred = 0, int threads = 1024);
+void launch_forced(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, const void* fin,
+                   void* fout, int level, sbot_stream_t s);
 void launch_force_sum(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, int steps,
                       sbot_stream_t s);
 void launch_ibm_geom(int storage, const DevPool& P, const int* inst_list, const int* pn, int cap, int steps,
@@ -213,7 +215,10 @@ int storage_bytes(int storage);
 // ---------------------------------------------------------------------------
 #define STEP_MAX_PHASES 512
 #define STEP_MAX_DEPS 8
-enum { PH_POSE = 0, PH_GEOM, PH_C2F, PH_FUSED, PH_IBM, PH_FSUM };
+enum { PH_POSE = 0, PH_GEOM, PH_C2F, PH_FUSED, PH_IBM, PH_FSUM, PH_FORCED };
+// storage of as many bytes (FP64): the step kernel's IBM leaves its cells' collision to
+// a phase of their own (ibm_run's LIST)
+constexpr int STEP_LIST_BYTES = 8;
 struct StepPhase {
     int kind;         // PH_*
     int bulk;         // 1: bulk queue (no dependencies); 0: critical queue
@@ -224,6 +229,7 @@ struct StepPhase {
     int count_idx;    // its length: index in the device count array
     int fold;         // PH_FUSED: its cells next to the finer region also write the finer level's halo (in ffine)
     int arg;          // PH_GEOM, PH_IBM: finest step of the coarse step; PH_FSUM: finest steps per coarse step;
+                      // PH_FORCED: tasks per body;
                       // PH_FUSED: 1 to keep one cell per thread (blocks whose pulls merge fine values)
     int ndep;
     int dep[STEP_MAX_DEPS];   // the phases this one waits for (all earlier; a bulk phase waits for none)

@@ -11,6 +11,8 @@
 //             inside the coarse pull)
 //   PH_IBM    multi-direct forcing of the bodies on their finest level (Sec. 2.2)
 //   PH_FSUM   the FP64 force and moment sums of the coarse step (Eq. 16)
+//   PH_FORCED FP64: the forced collision of the bodies' stencil cells, after the
+//             IBM and the sweep of its sub-step (ibm_run's LIST)
 // Every phase is cut into tasks of one thread block.  A phase may start once
 // every task of the phases it depends on has finished: each phase has a
 // counter of finished tasks, raised by one reduction with release semantics
@@ -146,7 +148,8 @@ __device__ int step_ntasks(const DevPool& P, const StepArgs& A, const StepPhase&
         const int per = T >= B * B ? T / (B * B) : 1;
         return (n + per - 1) / per;
     }
-    case PH_FSUM: return n * ph.arg;
+    case PH_FSUM:
+    case PH_FORCED: return n * ph.arg;
     default: return n;  // one body per task
     }
 }
@@ -245,8 +248,9 @@ __device__ void step_task(const DevPool& P, const StepArgs& A, const StepPhase& 
     switch (ph.kind) {
     case PH_FUSED: step_fused<S, C, B, COLL, VEC>(P, A, ph, local, grid, key, gate); break;
     case PH_IBM:
-        ibm_run<S, C, COLL>(P, list[local], step_buf<S>(A, ph.fin), step_buf<S>(A, ph.fout), ph.level, 0, 1, ph.arg,
-                            smraw, sh, gate, await, swept);
+        ibm_run<S, C, COLL, sizeof(S) == STEP_LIST_BYTES, true>(P, list[local], step_buf<S>(A, ph.fin),
+                                                                step_buf<S>(A, ph.fout), ph.level, 0, 1, ph.arg, smraw,
+                                                                sh, gate, await, swept);
         break;
     default: {
         if (!gate(false)) return;
@@ -260,6 +264,11 @@ __device__ void step_task(const DevPool& P, const StepArgs& A, const StepPhase& 
         }
         case PH_GEOM: ibm_geom_run<C>(P, list[local], ph.arg, smraw, sh); break;
         case PH_POSE: pose_run(P, list[local]); break;
+        case PH_FORCED:
+            if constexpr (sizeof(S) == STEP_LIST_BYTES)
+                ibm_forced_run<S, C, COLL>(P, list[local / ph.arg], step_buf<S>(A, ph.fin), step_buf<S>(A, ph.fout),
+                                           ph.level, local % ph.arg, ph.arg);
+            break;
         case PH_FSUM: force_sum_run<C>(P, list[local / ph.arg], local % ph.arg, sh.red); break;
         default: break;
         }
@@ -365,8 +374,13 @@ __device__ bool wait_until(const DevPool& P, const StepArgs& A, R&& ready) {
 // kernel without it: the vector sweep's registers make the rest spill
 // (immersed cylinder in a cavity 36.2 -> 32.4 us per step without it, D = 40
 // cylinder 50.5 -> 49.8).
+// FP64: the register count follows the thread blocks per SM asked for here.  One for
+// blocks of 16 and 32 (198 to 212 registers with the vector sweep, no spills; left
+// to the compiler it took 128 and spilled: 1024^2 220 -> 237 us per step, with the LES
+// collision 362 -> 406), whose FP64 work fills the pipe from one; two for blocks of 8.
+#define STEP_MIN_BLOCKS(S, B) (sizeof(S) == 8 ? ((B) == 8 ? 2 : 1) : 0)
 template <class S, class C, int B, int COLL, bool VEC>
-__global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS) k_step(const __grid_constant__ DevPool P, const __grid_constant__ StepArgs A) {
+__global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS, STEP_MIN_BLOCKS(S, B)) k_step(const __grid_constant__ DevPool P, const __grid_constant__ StepArgs A) {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ IbmShared sh;
     __shared__ int ntask[STEP_MAX_PHASES];   // tasks of each phase at this launch

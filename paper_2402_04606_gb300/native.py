@@ -289,7 +289,7 @@ class _InstanceCalls:
         return np.ascontiguousarray(buf[:, :n.value].T)
 
 
-PHASE_KINDS = ("pose", "ibm_geometry", "c2f_copy", "sweep", "ibm", "force_sums")
+PHASE_KINDS = ("pose", "ibm_geometry", "c2f_copy", "sweep", "ibm", "force_sums", "forced_cells")
 
 
 def _step_trace(obj) -> list:

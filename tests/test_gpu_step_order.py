@@ -130,3 +130,50 @@ def test_more_bodies_than_thread_blocks():
     assert np.array_equal(res[0][0], res[1][0])
     for x, y in zip(res[0][1], res[1][1]):
         assert np.array_equal(x, y) and np.array_equal(x, res[0][1][0])
+
+
+def wide_ellipse(storage):
+    """140 cells long on blocks of 8: 18 blocks, more than the IBM's slot table has a side"""
+    spec = wl.wing(c=140, levels=2, re=200.0, n_markers=230, block=8, domain_chords=3.0, storage=storage,
+                   thickness=10.0 / 140.0, heave_chords=0.0)
+    spec.body.motion = 0
+    spec.body.alpha_mean = 0.0
+    spec.margin = (0.0, 10.0) + (0.0,) * 6
+    spec.retag = 0
+    spec.init, spec.tgv_u0 = "tgv", 0.02
+    return spec
+
+
+def small_wing(storage):
+    spec = wl.wing(c=16, levels=3, re=100.0, n_markers=50, block=8, domain_chords=8.0, storage=storage,
+                   heave_chords=1.0)
+    spec.body.period = 400.0
+    spec.margin = (0.0, 14.0, 6.0) + (0.0,) * 5
+    return spec
+
+
+FORCED = {"wide": wide_ellipse, "wing": small_wing, "wing mrt": lambda st: wl.with_mrt(small_wing(st)),
+          "wing les": lambda st: wl.with_les(small_wing(st)),
+          "few cells": lambda st: wl.cylinder(D=10, levels=2, block=8, storage=st, n_markers=3)}
+
+
+@pytest.mark.parametrize("storage", [wl.F64, wl.F32, wl.BF16DEV])
+@pytest.mark.parametrize("name", list(FORCED))
+def test_forced_cells_collided_apart(name, storage):
+    """the collision of the cells a body forces: a launch of its own in the graphs, a phase of its own in FP64, by the
+    IBM's thread block in the other storage kinds"""
+    spec, steps = FORCED[name](storage), 20
+    pops, forces = run(spec, 1, steps, -1)
+    gp, gf = run(spec, 0, steps, -1)
+    for a, b in zip(pops, gp):
+        assert np.array_equal(a, b)
+    assert np.array_equal(forces, gf)
+    if storage != wl.F64:
+        return
+    o = init_oracle(oracle_from_spec(spec), spec)
+    o.step(steps)
+    for l in range(spec.levels):
+        m = o.types(l) == 1
+        assert rel_l2(pops[l][:, m], o.populations(l)[:, m]) <= 1e-12
+    fo = o.forces()
+    np.testing.assert_allclose(forces[:, :2], fo[:, :2], rtol=1e-10, atol=1e-11 * np.abs(fo[:, :2]).max())

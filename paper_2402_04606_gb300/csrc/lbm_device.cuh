@@ -2047,8 +2047,7 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
             }
         }
     }
-    const int rest = REG ? tid + nt : tid;  // the thread's first cell that is not in registers
-    for (int ci = rest; ci < ncell; ci += nt) {
+    for (int ci = REG ? tid + nt : tid; ci < ncell; ci += nt) {
         C v[9], inv;
         IbmV2<C> u;
         moments(ci, v, u, inv);
@@ -2116,7 +2115,7 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
             u0.y += sy * inv0;
             cu[tid] = u0;
         }
-        for (int ci = rest; ci < ncell; ci += nt) {
+        for (int ci = REG ? tid + nt : tid; ci < ncell; ci += nt) {
             C sx = 0, sy = 0;
             const int b1 = cst[ci + 1];
             for (int e = cst[ci]; e < b1; e++) {

@@ -84,6 +84,7 @@ __device__ __forceinline__ int fused_items(bool vec, int T) {
 
 // the most list items whose blocks' data a task of a sweep reads ahead
 #define STEP_META_MAX (STEP_MAX_THREADS / 64)
+static_assert(STEP_META_MAX < 16, "packed in step_fused's key");
 
 // How fused phase ph with n items is cut into tasks: `per` items per round and
 // `rounds` rounds per task, or (parts > 1) every item into `parts` tasks of its
@@ -176,7 +177,7 @@ __device__ __forceinline__ void for_cells(int n, int i0, int k, int BB, F&& fn) 
 // would not do: one list may be cut in two ways within a launch, as bulk tasks in
 // the first step and critical ones in the others).
 template <class S, class C, int B, int COLL, bool VEC, class G>
-__device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, int grid, int4& key,
+__device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, int grid, int2& key,
                            G& gate) {
     __shared__ SlotMeta<C> meta[STEP_META_MAX];
     const int n = A.counts[ph.count_idx];
@@ -194,10 +195,11 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
         // its cells: those of its items, or a part of one item's
         const int len = sh.parts > 1 ? B * B / sh.parts : (ne - i0) * B * B;
         const int c0 = sh.parts > 1 ? (local - i0 * sh.parts) * len : 0;
-        const bool held = key.x == ph.list_off && key.y == i0 && key.z == ne;
+        const int items = i0 << 4 | (ne - i0);  // (at most STEP_META_MAX of them)
+        const bool held = key.x == ph.list_off && key.y == items;
         if (!held && i0 + w < ne) load_meta<C>(P, list[i0 + w], ph.level, meta[w]);
         if (!gate(true)) return;
-        if (threadIdx.x == 0) key = make_int4(ph.list_off, i0, ne, 0);
+        if (threadIdx.x == 0) key = make_int2(ph.list_off, items);
         for (int c = c0 + threadIdx.x; c < c0 + len; c += T) {
             const SlotMeta<C>& m = meta[c / (B * B)];
             const int cell = c % (B * B);
@@ -238,7 +240,7 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
 // An IBM task waits before its stores for the sweep of its sub-step
 // (ph.after): await() by one warp, swept() by all after a barrier (ibm_run).
 template <class S, class C, int B, int COLL, bool VEC, class G, class G1, class G2>
-__device__ void step_task(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, int grid, int4& key,
+__device__ void step_task(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, int grid, int2& key,
                           unsigned char* smraw, IbmShared& sh, G& gate, G1& await, G2& swept) {
     const int* list = A.lists + ph.list_off;
     if (A.counts[ph.count_idx] <= 0) {  // the empty task of a phase with no work
@@ -392,7 +394,7 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS, STEP_
     // the scheduler's state lives in shared memory, so that no register is
     // held across a task (the vector sweep needs all of them)
     __shared__ int s_cmd, s_phase, s_local, s_last, s_ncp, s_nbulk, s_bulk_left, s_turn, s_next;
-    __shared__ int4 s_key;  // the sweep task whose blocks' data are held (step_fused)
+    __shared__ int2 s_key;  // whose blocks' data are held (step_fused)
     __shared__ int s_wait, s_go;  // the claimed critical phase to wait for (-1: none), the wait's outcome
     __shared__ int s_body[SBOT_MAXLEV + 1];  // first server of each group's bodies, their number
     const int tid = threadIdx.x, nph = A.nph;
@@ -414,7 +416,7 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS, STEP_
         s_body[SBOT_MAXLEV] = n <= A.max_servers ? n : 0;
         s_turn = 0;
         s_next = -1;
-        s_key = make_int4(-1, -1, -1, 0);
+        s_key = make_int2(-1, -1);
         sh.geo_inst = -1;
     }
     __syncthreads();

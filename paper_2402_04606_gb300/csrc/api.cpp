@@ -1719,7 +1719,13 @@ sbot_status step_persistent(sbot_ctx* c, int most, int* ran) {
                 (long long)c->wl[i].items.size() * c->B * c->B >= c->vec_min_cells)
                 A.any_vec = 1;
         }
-    A.max_servers = c->step_grid / 4;
+    // IBM servers for at most one thread block in 16 (9 bodies of one thread block per
+    // SM, 28 of three): beyond that the sweeps miss the SMs more than the bodies gain.
+    // us per step without servers / with: D = 40 cylinders, 8 of them 152 / 149, 16
+    // 263 / 271, 38 552 / 694; the mixed batch, 32 instances 1183 / 1387; D = 10
+    // cylinders (three thread blocks per SM), 8 of them 61.1 / 59.7, 32 137 / 141, 100
+    // 385 / 405.  A single body: k_step.
+    A.max_servers = c->step_grid / 16;
     for (int l = 0; l < SBOT_MAXLEV; l++) {
         const int gl = gl_of(l + 1, l);
         A.body_count[l] = (((c->groups >> l) & 1) && W_of(c, gl, LK_IBM).cap > 0) ? gl * LK_COUNT + LK_IBM : -1;

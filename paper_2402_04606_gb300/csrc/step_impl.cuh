@@ -401,11 +401,11 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS, STEP_
     StepCtl* ctl = A.ctl;
     constexpr unsigned FULL = 0xffffffffu;
 
-    // IBM servers: where there are at most max_servers bodies, the first
-    // thread blocks run one body's IBM each and nothing else, so that the IBM's
-    // code and its data stay in that SM's caches, a static body's geometry in
-    // its shared memory, and one step's IBM follows the last without a
-    // hand-over between SMs (D = 40 cylinder 54.7 -> 50.2 us per coarse step, the
+    // IBM servers: where there are at most max_servers bodies (the rule stands
+    // where the host sets it), the first thread blocks run one body's IBM each and
+    // nothing else, so that the IBM's code and its data stay in that SM's caches, a
+    // static body's geometry in its shared memory, and one step's IBM follows the
+    // last without a hand-over between SMs (D = 40 cylinder 54.7 -> 50.2 us per coarse step, the
     // D = 128 one 361 against 453 with the IBM handed out after the sweep's tasks)
     if (tid == 0) {
         int n = 0;

@@ -115,7 +115,7 @@ def tune(specs, storage: int | None = None, steps: int = 20, warmup: int = 5, bl
     (cells per thread: one below it, 4 in 32-bit and 8 in 16-bit storage
     above it), the shared-memory staged variant, programmatic dependent
     launch, the IBM's threads per body (256, 512, 1024), the vector kernel's
-    thread blocks (one per list group, or 2 waves of grid-stride blocks,
+    thread blocks (one per list group, or 2 waves of longer-lived blocks,
     against the default 8 waves), then the persistent
     step kernel at three vector-kernel thresholds of its own (the default,
     the graphs' best, never) and, at the best of those, its thread-block size

@@ -3,8 +3,7 @@
 //
 // Kernels
 //   k_fused        pull streaming (Eq. 10) + boundary rules + moments (Eq. 8) +
-//                  BGK collision with Guo forcing (Eqs. 3, 6, 7) on the leaf
-//                  blocks of one level; on fine-side halo blocks the same pull
+//                  BGK collision (Eqs. 6, 7) on the leaf blocks of one level; on fine-side halo blocks the same pull
 //                  without collision (Sec. 2.4 steps 3 and 5); the MRT and LES
 //                  collisions (Sec. 2.1) as variants.
 //   k_fused_v4     the same for large lists, 4 cells per thread (FP32, FP64);
@@ -14,8 +13,9 @@
 //   merge_fine     fine-to-coarse merge of the halo layers (Sec. 2.4 step 6),
 //                  evaluated inside the coarse pull (no kernel of its own).
 //   k_ibm          multi-direct-forcing immersed boundary on the finest level
-//                  (Sec. 2.2, Eqs. 11-16), one thread block per body;
-//                  k_ibm_geom its geometry for moving bodies, k_force_sum the
+//                  (Sec. 2.2, Eqs. 11-16), one thread block per body; k_forced
+//                  the collision of its stencil cells with their force (Guo
+//                  forcing, Eq. 3), over what the sweep wrote there; k_ibm_geom its geometry for moving bodies, k_force_sum the
 //                  Eq. 16 sums of a coarse step, k_pose the body poses.
 //   k_export / k_set_pre / k_checksum   state in and out.
 //

@@ -844,8 +844,8 @@ __device__ __forceinline__ void patch_force(const DevPool& P, const InstParams& 
 // ---------------------------------------------------------------------------
 // one cell of the fused step, scalar path: halo cells stream without
 // collision (Sec. 2.4 steps 3, 5); interior cells pull (Eq. 10 + boundary
-// rules) and collide (Eqs. 6-8).  No sweep reads an IBM force: the IBM collides
-// the cells it forces itself (ibm_run), after the sweep has written them.
+// rules) and collide (Eqs. 6-8).  No sweep reads an IBM force: the cells a body
+// forces are collided again with it (ibm_run), after the sweep has written them.
 // fhalo (non-null): the finer level's buffer whose halo cells inside this
 // level's blocks receive the post-collision populations of the coarse cell
 // that contains them (the coarse-to-fine copy of Sec. 2.4 step 2, done by the
@@ -879,7 +879,7 @@ __device__ __forceinline__ void fused_cell(const DevPool& P, M mt, const S* fin,
     C f[9];
     const int flags = mt.flags();
     const bool mailbox = (flags & SLOTF_MAILBOX) != 0;
-    unsigned links = 0;  // (SOLID: only in contexts holding a solid; the code costs every kernel that contains it)
+    unsigned links = 0;  // (SOLID: the graphs' kernel of contexts with a solid, and the step kernel, STEP_SOLID)
     const C* coef = nullptr;
     if constexpr (SOLID) {
         if (flags & SLOTF_SOLID) {
@@ -1442,11 +1442,11 @@ __device__ void pose_run(const DevPool& P, int inst) {
 // The iterations are bound by shared-memory wavefronts: with the lists read
 // from shared memory in every one, a cell phase of 600 cells issued about
 // 1200 of them (0.6 us).  So each thread keeps its first cell in registers
-// (list, velocity, force, 1/(2 rho), and its populations for the collision),
-// and an iteration reads only the force increments; and the smaller second part
-// lets bodies of up to about 430 markers run in the persistent kernel (the
-// paper's D = 128 cylinder, 402 markers: 456 us per coarse step in the
-// per-phase graphs, 302 there).
+// (list, velocity, force, 1/(2 rho), and its populations where it collides them
+// itself), and an iteration reads only the force increments; and the smaller
+// second part lets bodies of up to about 430 markers run in the persistent kernel
+// (the paper's D = 128 cylinder, 402 markers: 339 us per coarse step in the
+// per-phase graphs, 306 there).
 #define IBM_THREADS 1024
 #define IBM_RE 8  // list entries a thread keeps in registers (cells of bodies with markers a cell apart have 3 to 7)
 
@@ -2226,28 +2226,15 @@ __device__ void ibm_run(const DevPool& P, int inst, const S* fin, S* fout, int l
         }
     }
 }
-// the collision of one cell's populations f with the force (gx, gy).  LES in FP64: a
-// function of its own, so that the graphs' kernel and the step kernel round alike
-// (inlined, it contracted to different fmas in the two; the other collisions do
-// not, and called they cost a D = 40 cylinder's step 4 %)
-template <class S, class C, int COLL>
-__device__ __noinline__ void forced_apart(C* f, C om, C gx, C gy, const InstParams& ip) {
-    collide_k<COLL, C, true, DevTrait<S>::value, sizeof(S) == 4>(f, om, gx, gy, ip);
-}
-template <class S, class C, int COLL>
-__device__ __forceinline__ void forced_collision(C* f, C om, C gx, C gy, const InstParams& ip) {
-    if constexpr (sizeof(S) == STEP_LIST_BYTES && COLL == 2)
-        forced_apart<S, C, COLL>(f, om, gx, gy, ip);
-    else
-        collide_k<COLL, C, true, DevTrait<S>::value, sizeof(S) == 4>(f, om, gx, gy, ip);
-}
 // The forced collision of a body's stencil cells (LIST of ibm_run), part
 // `part` of `parts` of them by this thread block: pulled from fin again, with the
 // forces the patch holds, and stored in fout over what the sweep wrote there (an
 // inlet cell keeps the sweep's value: it is reset to the inlet state after
-// streaming).
+// streaming).  Not inlined: its registers stay out of the step kernel's sweeps, and
+// the graphs' kernel and the step kernel round alike (inlined, the LES collision in
+// FP64 contracted to different fmas in the two).
 template <class S, class C, int COLL>
-__device__ void ibm_forced_run(const DevPool& P, int inst, const S* fin, S* fout, int level, int part, int parts) {
+__device__ __noinline__ void ibm_forced_run(const DevPool& P, int inst, const S* fin, S* fout, int level, int part, int parts) {
     const InstParams& ip = P.inst[inst];
     const int entry = P.ist[inst].forced;
     if (entry < 0) return;
@@ -2269,7 +2256,7 @@ __device__ void ibm_forced_run(const DevPool& P, int inst, const S* fin, S* fout
             (gy == 0 && ip.bc[SIDE_S] == BCK_INLET) || (gy == nyl - 1 && ip.bc[SIDE_N] == BCK_INLET))
             continue;
         const IbmV2<C> g = F[ci];
-        forced_collision<S, C, COLL>(f, om, g.x, g.y, ip);
+        collide_k<COLL, C, true, DevTrait<S>::value, sizeof(S) == 4>(f, om, g.x, g.y, ip);
 #pragma unroll
         for (int q = 0; q < 9; q++) Sto<S>::template st<C>(fout, own + q * BB, q, f[q], ip.dref);
     }

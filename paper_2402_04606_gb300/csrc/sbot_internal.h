@@ -77,7 +77,8 @@ struct InstParams {
     int solid_blocks;                           // its blocks
     double ramp_as, ramp_rate, ramp_t1, t_ref;  // motion 3 (pitch-up ramp)
     double asym_xi, accel_frac;                 // motion 4 (triangular pitch)
-    void* patch;     // force patch, compute type, [2][patch_cap]
+    void* patch;     // compute type: the force field on the marker box at t = 0, [2][patch_cap]; later the forces
+                     // of the stencil cells, in pairs (ibm_forced_run)
     int patch_cap;   // cells of the force patch
     double* hist;    // force history ring, [SBOT_HIST_CAP][3]
     double* pose_tab;  // moving bodies: [pose_n][4] centre x, y, cos, sin of the pose at pose_k0 + i
@@ -259,7 +260,7 @@ struct StepArgs {
     int crit_items;           // > 0: at most this many list items per task of a critical fused phase
     int any_vec;              // 1: some sweep may take the vector mapping (by the host's list lengths)
     int fixed;                // 1: every task has a fixed owner (all instances have one level)
-    int max_servers;          // most thread blocks set apart for one body's IBM each (more bodies: no block is)
+    int max_servers;          // most thread blocks set apart for one body's IBM each (more bodies: none is)
     int body_count[SBOT_MAXLEV];  // per group, the index of its body list's length, -1 none
     // phase trace (nullptr: off): device ns of each phase's first task start
     // and last task end, its task count, and the launch's first start

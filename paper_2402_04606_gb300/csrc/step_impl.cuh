@@ -84,7 +84,6 @@ __device__ __forceinline__ int fused_items(bool vec, int T) {
 
 // the most list items whose blocks' data a task of a sweep reads ahead
 #define STEP_META_MAX (STEP_MAX_THREADS / 64)
-static_assert(STEP_META_MAX < 16, "packed in step_fused's key");
 
 // How fused phase ph with n items is cut into tasks: `per` items per round and
 // `rounds` rounds per task, or (parts > 1) every item into `parts` tasks of its
@@ -171,11 +170,12 @@ __device__ __forceinline__ void for_cells(int n, int i0, int k, int BB, F&& fn) 
 // their types, children) into shared memory, which it may do before the
 // phases it depends on have finished: after the gate only the population
 // and force loads remain on its path.
-// key: whose blocks' data the shared memory holds: the list and the items (a
-// thread block of a launch of fixed owners runs the same task in every step, and
-// reads them once; elsewhere it may draw the same items again.  The task's number
-// would not do: one list may be cut in two ways within a launch, as bulk tasks in
-// the first step and critical ones in the others).
+// key: which task's blocks' data the shared memory holds (a thread block of a
+// launch of fixed owners runs the same task in every step, and reads them once;
+// there a list is cut the same way in every phase, which elsewhere it is not: a
+// level-0 list is bulk in the first step and critical in the others.  A key of the
+// items themselves would hold them there too, and gained a D = 128 cylinder 0.7 %,
+// but cost every launch registers: 4096^2 in FP32 200.6 -> 204.3 us per step).
 template <class S, class C, int B, int COLL, bool VEC, class G>
 __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase& ph, int local, int grid, int2& key,
                            G& gate) {
@@ -195,11 +195,10 @@ __device__ void step_fused(const DevPool& P, const StepArgs& A, const StepPhase&
         // its cells: those of its items, or a part of one item's
         const int len = sh.parts > 1 ? B * B / sh.parts : (ne - i0) * B * B;
         const int c0 = sh.parts > 1 ? (local - i0 * sh.parts) * len : 0;
-        const int items = i0 << 4 | (ne - i0);  // (at most STEP_META_MAX of them)
-        const bool held = key.x == ph.list_off && key.y == items;
+        const bool held = A.fixed && key.x == ph.list_off && key.y == local;
         if (!held && i0 + w < ne) load_meta<C>(P, list[i0 + w], ph.level, meta[w]);
         if (!gate(true)) return;
-        if (threadIdx.x == 0) key = make_int2(ph.list_off, items);
+        if (A.fixed && threadIdx.x == 0) key = make_int2(ph.list_off, local);
         for (int c = c0 + threadIdx.x; c < c0 + len; c += T) {
             const SlotMeta<C>& m = meta[c / (B * B)];
             const int cell = c % (B * B);
@@ -405,8 +404,9 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : STEP_MAX_THREADS, STEP_
     // where the host sets it), the first thread blocks run one body's IBM each and
     // nothing else, so that the IBM's code and its data stay in that SM's caches, a
     // static body's geometry in its shared memory, and one step's IBM follows the
-    // last without a hand-over between SMs (D = 40 cylinder 54.7 -> 50.2 us per coarse step, the
-    // D = 128 one 361 against 453 with the IBM handed out after the sweep's tasks)
+    // last without a hand-over between SMs (D = 40 cylinder 54.7 -> 50.2 us per
+    // coarse step, the D = 128 one 361 against 453 with the IBM handed out after the
+    // sweep's tasks)
     if (tid == 0) {
         int n = 0;
         for (int g = 0; g < SBOT_MAXLEV; g++) {

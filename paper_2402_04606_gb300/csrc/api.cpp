@@ -1899,22 +1899,27 @@ sbot_status export_level(sbot_ctx* c, Inst& I, int level, int mode, double* cons
         }
     }
     cudaError_t e = cudaMemsetAsync(d, 0, bytes, c->s);
-    if (e == cudaSuccess) {
+    // an error of the steps leaves the caller's arrays as they are (the export pulls
+    // what the sweeps pulled, through the same tables, and finds none of its own)
+    const sbot_status st = check_device_error(c);
+    if (e == cudaSuccess && st == SBOT_OK) {
         DevPool P = pool_view(c);
         launch_export(c->storage, P, int_part(I, level), I.int_n[level], pre_buf(c, level), fine_buf(c, I, level), level,
                       I.coarse_step == 0 ? 1 : 0, nx, d, plane, mode, c->s);
         e = cudaGetLastError();
     }
-    // (an error leaves the caller's arrays as they are)
-    const sbot_status st = e == cudaSuccess ? check_device_error(c) : SBOT_OK;
+    // queued at once, so that the host's part of the copies (the caller's pages)
+    // runs beside the kernel: after a wait for it, 4096^2 fields took 23 ms
     for (int i = 0; i < n_out && e == cudaSuccess && st == SBOT_OK; i++)
         if (out[i]) e = cudaMemcpyAsync(out[i], (const char*)d + i * part, part, cudaMemcpyDeviceToHost, c->s);
+    int err = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->s);
     cudaError_t e2 = cudaStreamSynchronize(c->s);
     if (!keep) dfree(d);
     TRY(st);
     CK(e);
     CK(e2);
-    return SBOT_OK;
+    return report_device_error(c, err);
 }
 
 sbot_status validate_desc(const sbot_domain_desc* d, std::string& why) {

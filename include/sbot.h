@@ -226,12 +226,13 @@ sbot_status sbot_get_forces(sbot_ctx_t ctx, double* fx, double* fy, double* mz, 
 
 /* rho and the velocity sum_i c_i f_i / rho of the canonical (pre-collision)
  * state of level `level`, dense host arrays [ny_l][nx_l]; cells that are not
- * interior to that level are 0.  *n_cells_inout: capacity in, nx_l * ny_l out. */
+ * interior to that level are 0.  *n_cells_inout: capacity in, nx_l * ny_l out.
+ * An error of the steps before leaves the arrays as they are. */
 sbot_status sbot_get_fields(sbot_ctx_t ctx, int level, double* rho, double* ux, double* uy, int64_t* n_cells_inout);
 
 /* Canonical pre-collision populations of level `level`, dense host
  * [9][ny_l][nx_l] in FP64 (non-interior cells 0). *n_inout: capacity in
- * elements, 9 * nx_l * ny_l out. */
+ * elements, 9 * nx_l * ny_l out.  Errors as for sbot_get_fields. */
 sbot_status sbot_get_populations(sbot_ctx_t ctx, int level, double* f, int64_t* n_inout);
 
 /* Cell kinds of level `level`, dense [ny_l][nx_l]: 0 none, 1 interior,
@@ -278,8 +279,8 @@ sbot_status sbot_get_work(sbot_ctx_t ctx, int64_t* cell_updates, int64_t* fine_e
 /* Kernel timing of the hot path with CUDA events on the context stream.
  * sbot_set_profiling(ctx, mask): bit k enables kind k -- 0 fused
  * stream-collide, 1 coarse-to-fine halo copy, 2 fine-to-coarse merge (done
- * inside the coarse fused sweep, so it reports no launches of its own), 3 IBM;
- * 0 disables.  The events are recorded inside the step's CUDA graph (a new
+ * inside the coarse fused sweep, so it reports no launches of its own), 3 IBM
+ * with the collision of the cells it forces; 0 disables.  The events are recorded inside the step's CUDA graph (a new
  * mask recaptures it), which a profiled step captures on the context stream
  * alone: the kernels run one after another, so their times never overlap
  * (and add up to at most the profiled step); while enabled, sbot_step waits
